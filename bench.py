@@ -106,7 +106,7 @@ def stage_source_hash() -> str:
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("lbfs_stage.cu", "lbfs_internal.cuh"):
+    for f in ("lbfs_stage.cuh", "lbfs_stage.cu", "lbfs_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2511_10257_gb300", "csrc", f)) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         lines = [re.sub(r"//.*", "", ln).rstrip() for ln in src.splitlines()]

@@ -63,7 +63,8 @@ typedef struct lbfs_config {
                                 checked on the host (0: 40)                                */
     double  mg_tol;          /* relative residual ||b - A phi|| / ||b|| every solve must
                                 reach (0: 1e-13 FP64, 1e-6 mixed)                          */
-    int32_t tile;            /* stage-kernel tile shape id (see lbfs_autotune); 0: 32 x 8   */
+    int32_t tile;            /* stage-kernel strip shape id (see lbfs_autotune); 0: chosen
+                                from the cases' grids                                      */
     int32_t mg_warm_cycles;  /* refinement cycles available to the potential solve of each
                                 later step (0: 12 FP64, 3 mixed).  Each cycle ends with the
                                 residual of the corrected potential; once it meets mg_tol
@@ -230,24 +231,24 @@ lbfs_status lbfs_potential_pseudo_time(lbfs_ctx* ctx, int32_t case_id, int32_t i
  * bookkeeping, no counterpart in the paper. */
 int64_t lbfs_last_launch_count(const lbfs_ctx* ctx);
 
-/* Autotuner of the stage kernel's tile shape (no counterpart in the paper).  The tile
- * is a block's share of the grid; the halo is fixed at three cells by the stencil.
- * Times `reps` launches of each compiled tile shape on the context's current cases
- * (Runge-Kutta stage 2, which writes only a stage buffer, so the state is untouched),
+/* Autotuner of the stage kernel's strip shape (no counterpart in the paper).  A strip, 26
+ * columns by a number of rows, is one warp's share of the grid; the halo is fixed at three
+ * cells by the stencil.  Times `reps` launches of each strip shape on the context's current
+ * cases (Runge-Kutta stage 2, which writes only a stage buffer, so the state is untouched),
  * keeps the fastest (a shape with a higher id must be more than 2 % faster than the
  * best before it) for later steps and writes its id to *chosen (nullable).  ms
  * (nullable, n entries) receives the milliseconds per launch of each shape id < n.
- * Shapes: 0 32x8, 1 32x16, 2 64x8, 3 16x16, 4 64x4, 5 16x16 and 6 32x8 with registers
- * cut for a third resident block per SM, 7 16x16 and 8 32x8 with registers cut for a
- * fourth, 9 16x16 and 10 32x8 with a fourth block of 256 threads instead of 288 (the
- * cuts apply in mixed precision).  LBFS_EINVAL without a defined case or for reps < 1. */
+ * Shapes: 0 the library's own choice from the cases' grids, 1 to 12 strips of 128, 96, 64,
+ * 48, 32, 24, 16, 12, 8, 4, 2 and 1 rows.  Fields do not depend on the shape.  LBFS_EINVAL
+ * without a defined case or for reps < 1. */
 lbfs_status lbfs_autotune(lbfs_ctx* ctx, int32_t reps, int32_t* chosen, double* ms, int32_t n);
 
 /* Kernel timing (no counterpart in the paper).  While enabled, lbfs_step brackets
  * every launch with CUDA events on the context's stream and accumulates the elapsed
  * device time per kernel class: LBFS_TIMING_STAGE (the fused Runge-Kutta stage
- * kernel), LBFS_TIMING_POTENTIAL (the whole potential solve of a step),
- * LBFS_TIMING_FINALIZE (step-end statistics).  Enabling clears the accumulators; while
+ * kernel; its third launch also forms the step-end statistics), LBFS_TIMING_POTENTIAL (the
+ * whole potential solve of a step), LBFS_TIMING_FINALIZE (what a step launches after its
+ * last stage: nothing, an empty bracket).  Enabling clears the accumulators; while
  * enabled the step is never replayed from a graph.  lbfs_timing_read copies n (<= 3)
  * accumulated milliseconds and event-pair counts into caller-owned arrays (either may
  * be NULL). */

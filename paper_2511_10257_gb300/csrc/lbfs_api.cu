@@ -24,6 +24,8 @@ struct Slot {
     bool defined = false;
     lbfs_case_desc desc{};
     DevCase hd{};
+    StageCase<float> sf{};    // the stage kernel's view, in the context's precision
+    StageCase<double> sd{};
     void* block = nullptr;
 };
 
@@ -37,6 +39,7 @@ struct lbfs_ctx {
     std::vector<Slot> slots;
     DevCase* d_cases = nullptr;
     double* d_stats = nullptr;
+    void* d_stage_cases = nullptr;   // StageCase of every slot, in the context's precision
     TileRef* d_stage_tiles = nullptr;
     int n_stage_tiles = 0;
     std::vector<TileRef*> d_mg_tiles;
@@ -44,7 +47,6 @@ struct lbfs_ctx {
     std::vector<TileRef*> d_ft_tiles;   // fused V-cycle tiles per level
     std::vector<int> n_ft_tiles;
     std::vector<int> ft_small;          // per level: 16 x 8 fused tiles instead of 32 x 16
-    int* d_active = nullptr;
     int n_active = 0;
     int* d_pot = nullptr;
     int n_pot = 0;
@@ -64,7 +66,8 @@ struct lbfs_ctx {
     int mg_max_cycles = 0;
     int mg_warm_cycles = 0;
     int half = 0;          // every defined case has dts = 1/2
-    int tile = 0;          // stage-kernel tile shape id (config or autotuner)
+    int tile = 0;          // stage-kernel strip shape id (config or autotuner)
+    int rows = 0;          // rows of a strip, by the shape id or its rule
     bool pot_fresh = true; // a state was set since the last full potential solve
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
@@ -165,9 +168,6 @@ void harvest(lbfs_ctx* ctx) {
     ctx->ev_pending.clear();
 }
 
-int stage_tw(const lbfs_ctx* ctx) { return stage_tile_w(ctx->prec, ctx->tile); }
-int stage_th(const lbfs_ctx* ctx) { return stage_tile_h(ctx->prec, ctx->tile); }
-
 // Resolve the case parameters (Eq. 50 groups, mu_c coefficients, boundary flags).
 lbfs_status resolve(lbfs_ctx* ctx, const lbfs_case_desc& d, CaseParams& P) {
     std::memset(&P, 0, sizeof(P));
@@ -266,26 +266,74 @@ void fill_phys(const CaseParams& P, PhysT<R>& q) {
     q.Hes_lo = R(Hes - double(q.Hes_hi));
     q.L_hi = R(P.L);
     q.L_lo = R(P.L - double(q.L_hi));
+    q.rho_sg = q.rho_s - q.rho_g; q.rho_lg = q.rho_l - q.rho_g;
+    q.cp_sg = q.cp_s - q.cp_g; q.cp_lg = q.cp_l - q.cp_g;
+    q.mu_sg = q.mu_s - q.mu_g; q.mu_lg = q.mu_l - q.mu_g;
+    q.lam_sg = q.lam_s - q.lam_g; q.lam_lg = q.lam_l - q.lam_g; q.chi_lg = q.chi_l - q.chi_g;
+    q.m_Qg = -q.Q_g; q.m_cp_ref3 = R(-P.cp_ref / 3.0);
+    q.cp_ref3 = R(P.cp_ref / 3.0); q.inv_cps = R(1.0 / P.cp_s);
+    q.x_g = R(P.mobility / (P.Q_g * P.dts)); q.om_x_g = R(1) - q.x_g; q.beta2 = R(2.0 * P.beta); q.Qg3 = R(3.0 * P.Q_g);
+    q.mhd = R(-0.5 * P.dts); q.off = R(0.5 * (0.5 - P.dts)); q.inv_dt = R(1.0 / P.dt);
+}
+
+template <class R>
+void fill_stage(const DevCase& d, StageCase<R>& c) {
+    const CaseParams& P = d.P;
+    std::memset(&c, 0, sizeof(c));
+    fill_phys<R>(P, c.Q);
+    for (int k = 0; k < 3; ++k) {
+        c.He[k] = d.He[k];
+        c.W[k] = d.W[k];
+    }
+    c.phi = d.phi;
+    c.Fs_prev = d.Fs_prev;
+    c.Sdot = d.Sdot;
+    c.mu = d.lev[0].mu;
+    c.red = d.red;
+    c.red_groups = d.red_groups;
+    c.tickets = d.red_tickets;
+    c.stats = d.stats;
+    c.dt = P.dt;
+    c.solve_potential = P.solve_potential;
+    c.far_x = -2.0 * P.H0 * P.cos_t;
+    c.far_y = -2.0 * P.H0 * P.sin_t;
+    const double far[2] = {c.far_x, c.far_y};
+    for (int k = 0; k < 2; ++k) {
+        c.far_h[k] = (float)far[k];
+        c.far_l[k] = (float)(far[k] - (double)c.far_h[k]);
+    }
+    c.nx = P.nx; c.ny = P.ny; c.pitch = P.pitch;
+    c.periodic_x = P.periodic_x; c.periodic_y = P.periodic_y;
+    for (int w = 0; w < 4; ++w) {
+        c.thermal_dir[w] = P.thermal_dir[w];
+        c.mag_dir[w] = P.mag_dir[w];
+    }
 }
 
 // Upload the concatenated tile lists of all defined cases.
 lbfs_status rebuild(lbfs_ctx* ctx) {
     drop_graph(ctx);
-    const int TX = stage_tw(ctx), TY = stage_th(ctx);
     std::vector<TileRef> st;
-    std::vector<int> act, pot;
-    int depth = 0, coarsest = 0;
+    long long row_warps = 0;   // strips of one row's height over all cases
+    for (const Slot& s : ctx->slots)
+        if (s.defined) row_warps += (long long)((s.hd.P.nx + kStripW - 1) / kStripW) * s.hd.P.ny;
+    const int TX = kStripW, TY = stage_rows(ctx->prec, ctx->tile, row_warps, ctx->sm_count);
+    ctx->rows = TY;
+    std::vector<int> pot;
+    int active = 0, depth = 0, coarsest = 0;
     int half = 1;
     for (int c = 0; c < (int)ctx->slots.size(); ++c) {
         Slot& s = ctx->slots[c];
         if (!s.defined) continue;
-        const int rt = ((s.hd.P.nx + TX - 1) / TX) * ((s.hd.P.ny + TY - 1) / TY);
-        if (rt != s.hd.red_tiles) {
-            s.hd.red_tiles = rt;
-            if (cudaMemcpy(ctx->d_cases + c, &s.hd, sizeof(DevCase), cudaMemcpyHostToDevice) != cudaSuccess)
+        const int strips = ((s.hd.P.nx + TX - 1) / TX) * ((s.hd.P.ny + TY - 1) / TY);
+        if (strips != s.sf.strips) {
+            s.sf.strips = s.sd.strips = strips;
+            const void* sc = ctx->prec == 0 ? (const void*)&s.sd : (const void*)&s.sf;
+            const size_t scb = ctx->prec == 0 ? sizeof(s.sd) : sizeof(s.sf);
+            if (cudaMemcpy(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb, cudaMemcpyHostToDevice) != cudaSuccess)
                 return fail(ctx, LBFS_ECUDA, "case table update failed");
         }
-        act.push_back(c);
+        ++active;
         if (s.hd.P.dts != 0.5) half = 0;
         int slot = 0;
         for (int y = 0; y < s.hd.P.ny; y += TY)
@@ -337,8 +385,7 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
     if (!upload((void**)&ctx->d_stage_tiles, st.data(), st.size() * sizeof(TileRef)) ||
-        !upload((void**)&ctx->d_active, act.data(), act.size() * sizeof(int)) ||
-        !upload((void**)&ctx->d_pot, pot.data(), pot.size() * sizeof(int)))
+    !upload((void**)&ctx->d_pot, pot.data(), pot.size() * sizeof(int)))
         return fail(ctx, LBFS_ENOMEM, "tile list upload failed");
     for (auto* p : ctx->d_mg_tiles) dfree(ctx, p);
     for (auto* p : ctx->d_ft_tiles) dfree(ctx, p);
@@ -354,7 +401,7 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         ctx->n_ft_tiles[L] = (int)ft[L].size();
     }
     ctx->n_stage_tiles = (int)st.size();
-    ctx->n_active = (int)act.size();
+    ctx->n_active = active;
     ctx->n_pot = (int)pot.size();
     ctx->max_depth = depth;
     ctx->coarsest_cells = coarsest;
@@ -540,6 +587,19 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
     return LBFS_OK;
 }
 
+// stage k of every case
+cudaError_t stage(lbfs_ctx* ctx, int k) {
+    const Slot* one = nullptr;
+    if (ctx->n_active == 1)
+        for (const Slot& s : ctx->slots)
+            if (s.defined) one = &s;
+    if (ctx->prec == 0)
+        return launch_stage<double>(ctx->half, one ? &one->sd : nullptr, static_cast<StageCase<double>*>(ctx->d_stage_cases),
+                                    ctx->d_stage_tiles, ctx->n_stage_tiles, ctx->rows, k, ctx->stream);
+    return launch_stage<float>(ctx->half, one ? &one->sf : nullptr, static_cast<StageCase<float>*>(ctx->d_stage_cases),
+                               ctx->d_stage_tiles, ctx->n_stage_tiles, ctx->rows, k, ctx->stream);
+}
+
 lbfs_status one_step(lbfs_ctx* ctx) {
     cudaEvent_t t0 = tic(ctx);
     lbfs_status r = potential_solve(ctx);
@@ -547,12 +607,10 @@ lbfs_status one_step(lbfs_ctx* ctx) {
     toc(ctx, LBFS_TIMING_POTENTIAL, t0);
     for (int k = 0; k < 3; ++k) {
         cudaEvent_t t1 = tic(ctx);
-        LK(launch_stage(ctx->prec, ctx->tile, ctx->half, ctx->d_cases, ctx->d_stage_tiles,
-                        ctx->n_stage_tiles, k, ctx->stream));
+        LK(stage(ctx, k));
         toc(ctx, LBFS_TIMING_STAGE, t1);
     }
-    cudaEvent_t t2 = tic(ctx);
-    LK(launch_step_finalize(ctx->prec, ctx->d_cases, ctx->d_active, ctx->n_active, ctx->stream));
+    cudaEvent_t t2 = tic(ctx);   // (the step-end statistics are part of stage 3)
     toc(ctx, LBFS_TIMING_FINALIZE, t2);
     return LBFS_OK;
 }
@@ -638,9 +696,10 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
         ctx->own_stream = true;
     }
     ctx->d_cases = static_cast<DevCase*>(dalloc(ctx, sizeof(DevCase) * cfg->max_cases));
+    ctx->d_stage_cases = dalloc(ctx, (ctx->prec == 0 ? sizeof(StageCase<double>) : sizeof(StageCase<float>)) * cfg->max_cases);
     ctx->d_stats = static_cast<double*>(dalloc(ctx, sizeof(double) * kStatN * cfg->max_cases));
     ctx->d_flag = static_cast<int*>(dalloc(ctx, 256));
-    if (!ctx->d_cases || !ctx->d_stats || !ctx->d_flag ||
+    if (!ctx->d_cases || !ctx->d_stage_cases || !ctx->d_stats || !ctx->d_flag ||
         cudaMallocHost(&ctx->h_flag, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_stats, sizeof(double) * kStatN * cfg->max_cases) != cudaSuccess) {
         lbfs_destroy(ctx);
@@ -697,15 +756,8 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
                     "the potential's coarsest level would exceed 4096 cells (a periodic axis whose size "
                     "halves to an odd number early, or an extreme aspect ratio)");
     hd.nlev = nlev;
-    fill_phys<float>(P, hd.qf);
-    fill_phys<double>(P, hd.qd);
-    const int TX = stage_tw(ctx), TY = stage_th(ctx);
-    hd.red_tiles = ((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY);
-    int red_cap = 0;  // partial-sum slots for the tile shape with the most tiles
-    for (int t = 0; t < stage_tile_shapes(); ++t) {
-        const int w = stage_tile_w(ctx->prec, t), h = stage_tile_h(ctx->prec, t);
-        red_cap = std::max(red_cap, ((P.nx + w - 1) / w) * ((P.ny + h - 1) / h));
-    }
+    // partial-sum slots for the lowest strips
+    const int red_cap = ((P.nx + kStripW - 1) / kStripW) * ((P.ny + kStageMinRows - 1) / kStageMinRows);
     hd.mg_tiles = ((P.nx + kMgTX - 1) / kMgTX) * ((P.ny + kMgTY - 1) / kMgTY);
     // one device block per case
     const size_t rs = ctx->prec == 0 ? sizeof(double) : sizeof(float);
@@ -718,10 +770,7 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     };
     for (int k = 0; k < 3; ++k) {
         add(&hd.He[k], cells * sizeof(double));
-        add(&hd.p[k], cells * rs);
-        add(&hd.mx[k], cells * rs);
-        add(&hd.my[k], cells * rs);
-        add(&hd.C[k], cells * rs);
+        add(&hd.W[k], cells * 4 * rs);
     }
     if (ctx->prec == 0) {
         add((void**)&hd.phi64, cells * sizeof(double));
@@ -739,7 +788,10 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
         add(&hd.lev[L].e, lc * rs);
         add(&hd.lev[L].r, lc * rs);
     }
+    const int red_groups = (red_cap + kStageGroup - 1) / kStageGroup;
     add((void**)&hd.red, (size_t)red_cap * kRedN * sizeof(double));
+    add((void**)&hd.red_groups, (size_t)red_groups * kRedN * sizeof(double));
+    add((void**)&hd.red_tickets, (size_t)(1 + red_groups) * sizeof(unsigned));
     add((void**)&hd.mg_red, (size_t)hd.mg_tiles * 2 * sizeof(double));
     add((void**)&hd.chunk, (size_t)kFinChunks * (kRedN + 2) * sizeof(double));
     add((void**)&hd.tickets, 2 * sizeof(unsigned));
@@ -754,8 +806,18 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     hd.stats = ctx->d_stats + (size_t)id * kStatN;
     s.hd = hd;
     s.desc = *desc;
+    const void* sc = &s.sf;
+    size_t scb = sizeof(s.sf);
+    if (ctx->prec == 0) {
+        fill_stage<double>(hd, s.sd);
+        sc = &s.sd;
+        scb = sizeof(s.sd);
+    } else {
+        fill_stage<float>(hd, s.sf);
+    }
     CK(cudaMemsetAsync(s.block, 0, off, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_cases + id, &s.hd, sizeof(DevCase), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(static_cast<char*>(ctx->d_stage_cases) + id * scb, sc, scb, cudaMemcpyHostToDevice, ctx->stream));
     double st0[kStatN];
     for (double& v : st0) v = 0.0;
     st0[ST_T_FREEZE] = -1.0;
@@ -962,12 +1024,10 @@ lbfs_status lbfs_autotune(lbfs_ctx* ctx, int32_t reps, int32_t* chosen, double* 
         if (r != LBFS_OK) return r;
         // Runge-Kutta stage 2 reads sets 0 and 1 and dF_s/dt and writes only the stage
         // buffer 2, so timing it leaves the state untouched
-        CK(launch_stage(ctx->prec, t, ctx->half, ctx->d_cases, ctx->d_stage_tiles, ctx->n_stage_tiles, 1,
-                        ctx->stream));
+        CK(stage(ctx, 1));
         CK(cudaEventRecord(a, ctx->stream));
         for (int k = 0; k < reps; ++k)
-            CK(launch_stage(ctx->prec, t, ctx->half, ctx->d_cases, ctx->d_stage_tiles, ctx->n_stage_tiles, 1,
-                            ctx->stream));
+            CK(stage(ctx, 1));
         CK(cudaEventRecord(b, ctx->stream));
         CK(cudaEventSynchronize(b));
         float el = 0.f;
@@ -1023,8 +1083,8 @@ void lbfs_destroy(lbfs_ctx* ctx) {
     for (Slot& s : ctx->slots) free_slot(ctx, s);
     for (auto* p : ctx->d_mg_tiles) dfree(ctx, p);
     for (auto* p : ctx->d_ft_tiles) dfree(ctx, p);
+    dfree(ctx, ctx->d_stage_cases);
     dfree(ctx, ctx->d_stage_tiles);
-    dfree(ctx, ctx->d_active);
     dfree(ctx, ctx->d_pot);
     dfree(ctx, ctx->d_cases);
     dfree(ctx, ctx->d_stats);

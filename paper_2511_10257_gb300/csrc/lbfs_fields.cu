@@ -32,10 +32,10 @@ __global__ void k_init(const DevCase* __restrict__ dc, InitArgs a) {
     const double He = cp * a.T_init + P.L;
     const size_t k = (size_t)j * P.pitch + i;
     he_set<R>(dc->He[0], k, He);
-    static_cast<R*>(dc->p[0])[k] = R(0);
-    static_cast<R*>(dc->mx[0])[k] = R(0);
-    static_cast<R*>(dc->my[0])[k] = R(0);
-    static_cast<R*>(dc->C[0])[k] = R(C);
+    typename Quad<R>::T w;
+    w.x = w.y = w.z = R(0);
+    w.w = R(C);
+    static_cast<typename Quad<R>::T*>(dc->W[0])[k] = w;
     phi_set<R>(dc, k, -P.H0 * (x * P.cos_t + y * P.sin_t));
     R T, Fl;
     invert_enthalpy<R, double>(P, He, R(C), T, Fl);
@@ -48,7 +48,7 @@ __global__ void k_mu_from_state(const DevCase* __restrict__ dc) {
     const CaseParams& P = dc->P;
     if (!cell_of(P.nx, P.ny, i, j)) return;
     const size_t k = (size_t)j * P.pitch + i;
-    const R C = static_cast<const R*>(dc->C[0])[k];
+    const R C = static_cast<const typename Quad<R>::T*>(dc->W[0])[k].w;
     R T, Fl;
     invert_enthalpy<R, double>(P, he_get<R>(dc->He[0], k), C, T, Fl);
     static_cast<R*>(dc->lev[0].mu)[(size_t)j * dc->lev[0].pitch + i] =
@@ -56,14 +56,14 @@ __global__ void k_mu_from_state(const DevCase* __restrict__ dc) {
 }
 
 template <class R>
-__device__ __forceinline__ R C_at(const CaseParams& P, const R* C, int i, int j) {
+__device__ __forceinline__ R C_at(const CaseParams& P, const typename Quad<R>::T* W, int i, int j) {
     // C with the wall ghost rule (wetting; zero gradient at 90 degrees) or periodic wrap
     bool wall = false;
     if (i < 0) { wall = !P.periodic_x; i = P.periodic_x ? i + P.nx : 0; }
     if (i >= P.nx) { wall = !P.periodic_x; i = P.periodic_x ? i - P.nx : P.nx - 1; }
     if (j < 0) { wall = wall || !P.periodic_y; j = P.periodic_y ? j + P.ny : 0; }
     if (j >= P.ny) { wall = wall || !P.periodic_y; j = P.periodic_y ? j - P.ny : P.ny - 1; }
-    const R c = C[(size_t)j * P.pitch + i];
+    const R c = W[(size_t)j * P.pitch + i].w;
     return wall ? c + R(P.wet) * c * (R(1) - c) : c;
 }
 
@@ -75,12 +75,13 @@ __global__ void k_derive(const DevCase* __restrict__ dc, uint32_t mask, double* 
     const size_t k = (size_t)j * P.pitch + i;
     const size_t N = (size_t)P.nx * P.ny, o = (size_t)j * P.nx + i;
     const double He = he_get<R>(dc->He[0], k);
-    const R* Cg = static_cast<const R*>(dc->C[0]);
-    const R C = Cg[k];
+    const typename Quad<R>::T* Wg = static_cast<const typename Quad<R>::T*>(dc->W[0]);
+    const typename Quad<R>::T w = Wg[k];
+    const R C = w.w;
     R T, Fl;
     invert_enthalpy<R, double>(P, He, C, T, Fl);
     const R rho = mixture(R(1) - Fl, C, P.rho_s, P.rho_l, P.rho_g);
-    const R mx = static_cast<const R*>(dc->mx[0])[k], my = static_cast<const R*>(dc->my[0])[k];
+    const R mx = w.y, my = w.z;
     int slot = 0;
     for (int f = 0; f < 13; ++f) {
         if (!(mask & (1u << f))) continue;
@@ -90,13 +91,13 @@ __global__ void k_derive(const DevCase* __restrict__ dc, uint32_t mask, double* 
         case 1: v = He; break;
         case 2: v = (double)T; break;
         case 3: v = (double)Fl; break;
-        case 4: v = (double)static_cast<const R*>(dc->p[0])[k]; break;
+        case 4: v = (double)w.x; break;
         case 5: v = (double)(mx * R(3) / rho); break;
         case 6: v = (double)(my * R(3) / rho); break;
         case 7: v = (double)C; break;
         case 8: {
-            const R lap = C_at<R>(P, Cg, i + 1, j) + C_at<R>(P, Cg, i - 1, j) + C_at<R>(P, Cg, i, j + 1) +
-                          C_at<R>(P, Cg, i, j - 1) - R(4) * C;
+            const R lap = C_at<R>(P, Wg, i + 1, j) + C_at<R>(P, Wg, i - 1, j) + C_at<R>(P, Wg, i, j + 1) +
+                          C_at<R>(P, Wg, i, j - 1) - R(4) * C;
             v = (double)(R(2) * R(P.beta) * C * (C - R(1)) * (R(2) * C - R(1)) - R(P.kappa) * lap);
             break;
         }
@@ -125,15 +126,13 @@ __global__ void k_diag_columns(const DevCase* __restrict__ dc, double* __restric
     const CaseParams& P = dc->P;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.nx) return;
-    const R* Cg = static_cast<const R*>(dc->C[0]);
-    const R* mxg = static_cast<const R*>(dc->mx[0]);
-    const R* myg = static_cast<const R*>(dc->my[0]);
+    const typename Quad<R>::T* Wg = static_cast<const typename Quad<R>::T*>(dc->W[0]);
     const void* Heg = dc->He[0];
     double h = 0.0, umax = 0.0, C_above = 0.0;
     bool top_found = false;
     for (int j = P.ny - 1; j >= 0; --j) {
         const size_t k = (size_t)j * P.pitch + i;
-        const double C = (double)Cg[k];
+        const double C = (double)Wg[k].w;
         if (C >= 0.5) {
             if (!top_found) {
                 top_found = true;
@@ -142,14 +141,14 @@ __global__ void k_diag_columns(const DevCase* __restrict__ dc, double* __restric
             double T, Fl;
             invert_enthalpy<double, double>(P, he_get<R>(Heg, k), C, T, Fl);
             const double rho = mixture<double>(1.0 - Fl, C, P.rho_s, P.rho_l, P.rho_g);
-            const double u = (double)mxg[k] * 3.0 / rho, v = (double)myg[k] * 3.0 / rho;
+            const double u = (double)Wg[k].y * 3.0 / rho, v = (double)Wg[k].z * 3.0 / rho;
             umax = fmax(umax, sqrt(u * u + v * v));
         }
         C_above = C;
     }
     double Q = 0.0;
     if (!P.periodic_y && P.thermal_dir[2]) {
-        const double C0 = (double)Cg[i];
+        const double C0 = (double)Wg[i].w;
         double T0, Fl0;
         invert_enthalpy<double, double>(P, he_get<R>(Heg, i), C0, T0, Fl0);
         const double lam = mixture<double>(1.0 - Fl0, C0, P.lam_s, P.lam_l, P.lam_g);
@@ -158,7 +157,7 @@ __global__ void k_diag_columns(const DevCase* __restrict__ dc, double* __restric
         if (P.ny >= 2) {
             const size_t k1 = (size_t)P.pitch + i;
             double T1, Fl1;
-            invert_enthalpy<double, double>(P, he_get<R>(Heg, k1), (double)Cg[k1], T1, Fl1);
+            invert_enthalpy<double, double>(P, he_get<R>(Heg, k1), (double)Wg[k1].w, T1, Fl1);
             slope = (-8.0 * Tw + 9.0 * T0 - T1) / 3.0;
         } else {
             slope = (T0 - Tw) / 0.5;
@@ -217,6 +216,7 @@ __global__ void k_store(const DevCase* __restrict__ dc, uint32_t mask, const dou
     if (!cell_of(P.nx, P.ny, i, j)) return;
     const size_t k = (size_t)j * P.pitch + i;
     const size_t N = (size_t)P.nx * P.ny, o = (size_t)j * P.nx + i;
+    typename Quad<R>::T* W = static_cast<typename Quad<R>::T*>(dc->W[0]) + k;
     int slot = 0;
     for (int f = 0; f < 13; ++f) {
         if (!(mask & (1u << f))) continue;
@@ -224,10 +224,10 @@ __global__ void k_store(const DevCase* __restrict__ dc, uint32_t mask, const dou
         switch (f) {
         case 0: phi_set<R>(dc, k, v); break;
         case 1: he_set<R>(dc->He[0], k, v); break;
-        case 4: static_cast<R*>(dc->p[0])[k] = R(v); break;
-        case 7: static_cast<R*>(dc->C[0])[k] = R(v); break;
-        case 10: static_cast<R*>(dc->mx[0])[k] = R(v); break;
-        case 11: static_cast<R*>(dc->my[0])[k] = R(v); break;
+        case 4: W->x = R(v); break;
+        case 7: W->w = R(v); break;
+        case 10: W->y = R(v); break;
+        case 11: W->z = R(v); break;
         case 12: static_cast<R*>(dc->Fs_prev)[k] = R(v); break;
         default: break;
         }
@@ -252,11 +252,11 @@ __global__ void k_stats_init(const DevCase* __restrict__ dc) {
     DSum<R> acc[5];
     for (int q = 0; q < 5; ++q) acc[q] = DSum<R>::zero();
     const HS* He = static_cast<const HS*>(dc->He[0]);
-    const R* Cg = static_cast<const R*>(dc->C[0]);
+    const typename Quad<R>::T* Wg = static_cast<const typename Quad<R>::T*>(dc->W[0]);
     for (int j = j0; j < j1; ++j)
         for (int i = threadIdx.x; i < P.nx; i += blockDim.x) {
             const size_t k = (size_t)j * P.pitch + i;
-            const R C = Cg[k];
+            const R C = Wg[k].w;
             R T, Fl;
             invert_enthalpy<R, double>(P, he_value(He[k]), C, T, Fl);
             acc[0].add(C);
@@ -291,70 +291,6 @@ __global__ void k_stats_init(const DevCase* __restrict__ dc) {
     st[ST_N_DROP] = a[3];
     st[ST_Q_L] = a[3] > 0 ? a[4] / a[3] : 0.0;
     st[ST_QL_PREV] = st[ST_Q_L];
-}
-
-// step end: fixed-order sum of the stage-tile partials (FP64, or FP32 pairs in mixed
-// precision), Eq. 51 liquid-fraction measure, freezing time (first t with Q_L >= 0.99,
-// linear between steps).  kFinChunks blocks per case each sum a fixed contiguous range
-// of tiles; the block that finishes last (a ticket, no waiting) sums the chunk sums
-// in chunk order and updates the statistics, so the result does not depend on which
-// block is last.
-template <class R>
-__global__ void k_step_finalize(const DevCase* __restrict__ cases, const int* __restrict__ ids) {
-    using Slot = typename DSum<R>::Slot;
-    __shared__ Slot sh[32];
-    __shared__ bool last;
-    const DevCase* dc = cases + ids[blockIdx.y];
-    const int T = dc->red_tiles, c = blockIdx.x;
-    const int t0 = (int)((long long)T * c / kFinChunks), t1 = (int)((long long)T * (c + 1) / kFinChunks);
-    const Slot* red = static_cast<const Slot*>(dc->red);
-    DSum<R> acc[kRedN];
-    for (int q = 0; q < kRedN; ++q) acc[q] = DSum<R>::zero();
-    for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x)
-        for (int q = 0; q < kRedN; ++q) acc[q].add(DSum<R>::of(red[(size_t)t * kRedN + q]));
-    for (int q = 0; q < kRedN; ++q) acc[q] = block_sum0<R>(acc[q], sh);
-    Slot* ch = static_cast<Slot*>(dc->chunk);
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < kRedN; ++q) ch[c * kRedN + q] = acc[q].slot();
-        __threadfence();
-        last = atomicAdd(&dc->tickets[0], 1u) == (unsigned)(kFinChunks - 1);
-    }
-    __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
-    __threadfence();
-    // the chunk sums, one per lane, combined by a fixed shuffle tree (the same order
-    // whichever block is last)
-    static_assert(kFinChunks <= 32, "one chunk per lane");
-    const int lane = threadIdx.x;
-    double a[kRedN];
-    for (int q = 0; q < kRedN; ++q) {
-        DSum<R> v = lane < kFinChunks ? DSum<R>::of(ld_cg(&ch[lane * kRedN + q])) : DSum<R>::zero();
-        for (int o = 16; o > 0; o >>= 1) v.shfl_add(o);
-        a[q] = v.value();
-    }
-    if (lane != 0) return;
-    dc->tickets[0] = 0u;
-    double* st = dc->stats;
-    const double dt = dc->P.dt;
-    st[ST_SUM_C] = a[0];
-    st[ST_SUM_HE] = a[1];
-    st[ST_SUM_FL_DROP] = a[2];
-    st[ST_N_DROP] = a[3];
-    const double QL = a[3] > 0.0 ? a[4] / a[3] : 0.0;
-    st[ST_Q_L] = QL;
-    if (a[5] > 0.0) st[ST_NONFINITE] = 1.0;
-    st[ST_T] += dt;
-    st[ST_STEP] += 1.0;
-    if (st[ST_T_FREEZE] < 0.0 && QL >= 0.99) {
-        const double q0 = st[ST_QL_PREV];
-        st[ST_T_FREEZE] = (st[ST_T] - dt) + dt * (0.99 - q0) / (QL - q0);
-    }
-    st[ST_QL_PREV] = QL;
-    if (dc->P.solve_potential) {
-        st[ST_POT_RESID_MAX] = fmax(st[ST_POT_RESID_MAX], st[ST_POT_RESID]);
-        st[ST_POT_CYCLES_SUM] += st[ST_POT_CYCLES];
-    }
-    st[ST_STEPS_CALL] += 1.0;
 }
 
 }  // namespace
@@ -401,14 +337,6 @@ cudaError_t launch_stats_init(int prec, const DevCase* d, int nx, int ny, cudaSt
     (void)ny;
     if (prec == 0) k_stats_init<double><<<kFinChunks, 512, 0, st>>>(d);
     else k_stats_init<float><<<kFinChunks, 512, 0, st>>>(d);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_step_finalize(int prec, const DevCase* cases, const int* ids, int ncases, cudaStream_t st) {
-    if (ncases <= 0) return cudaSuccess;
-    const dim3 grid(kFinChunks, ncases);
-    if (prec == 0) k_step_finalize<double><<<grid, 256, 0, st>>>(cases, ids);
-    else k_step_finalize<float><<<grid, 256, 0, st>>>(cases, ids);
     return cudaGetLastError();
 }
 

@@ -47,6 +47,25 @@ struct PhysT {
     // the thresholds H_es = C_p,s T_m and L of Eq. 8 as (hi, lo) pairs of R: the exact
     // FP64 value is hi + lo to FP32-pair accuracy (lo = 0 in FP64)
     R Hes_hi, Hes_lo, L_hi, L_lo;
+    // what the stage kernel uses of the above, formed once: property differences g_s - g_g
+    // and g_l - g_g, C_p,ref/3, 1/C_p,s, tau_g - 1/2, 2 beta, 3 Q_g, -dts/2, (1/2 - dts)/2, 1/dt
+    R rho_sg, rho_lg, cp_sg, cp_lg, mu_sg, mu_lg, lam_sg, lam_lg, chi_lg;
+    R m_Qg, m_cp_ref3, om_x_g, cp_ref3, inv_cps, x_g, beta2, Qg3, mhd, off, inv_dt;
+};
+
+// p, rho c_s^2 u, rho c_s^2 v and C of one cell: one vector load or store
+struct alignas(32) Quad64 {
+    double x, y, z, w;
+};
+template <class R>
+struct Quad;
+template <>
+struct Quad<float> {
+    using T = float4;
+};
+template <>
+struct Quad<double> {
+    using T = Quad64;
 };
 
 struct MGLevel {
@@ -66,27 +85,47 @@ struct DevCase {
     CaseParams P;
     // state sets: 0 = W^n (and W^{n+1}), 1 and 2 = Runge-Kutta stage buffers
     void* He[3];      // HR precision (FP64 in both modes)
-    void* p[3];       // R precision
-    void* mx[3];
-    void* my[3];
-    void* C[3];
+    void* W[3];       // Quad<R>: p, rho c_s^2 u, rho c_s^2 v, C
     void* phi;        // potential read by the stage kernel (R); FP64 mode: the master
     double* phi64;    // FP64 mode: the master potential (== phi); mixed: unused
     double* phi_prev64;  // FP64 mode: the previous step's potential; mixed: unused
     float* phi_lo;    // mixed: low word of the master potential phi + phi_lo (FP32 pair)
     void* Fs_prev;    // R: F_s of the previous step, replaced by F_s^n in stage 1
     void* Sdot;       // R: lagged dF_s/dt of the current step, written by stage 1
-    PhysT<float> qf;
-    PhysT<double> qd;
     int nlev;
     MGLevel lev[kMaxLevels];
-    void* red;        // stage-tile partial sums, kRedN 8-byte DSum slots per tile
-    int red_tiles;    // number of stage tiles of this case
+    void* red;        // stage-strip partial sums, kRedN 8-byte DSum slots per strip
+    void* red_groups; // the same per group of strips
+    unsigned* red_tickets;
     void* mg_red;     // potential residual partial sums, 2 DSum slots per fine tile
     void* chunk;      // kFinChunks x (kRedN + 2) DSum slots: per-chunk sums of the partials
-    unsigned* tickets;  // [0] step-end, [1] residual: chunks done (the last one finalises)
+    unsigned* tickets;  // [0] set-up statistics, [1] residual: chunks done (the last one finalises)
     int mg_tiles;
     double* stats;    // kStatN FP64 slots
+};
+
+// What the stage kernel needs of one case.
+template <class R>
+struct StageCase {
+    PhysT<R> Q;
+    void* He[3];
+    void* W[3];
+    void* phi;
+    void* Fs_prev;
+    void* Sdot;
+    void* mu;         // the potential's fine-level coefficient (the fields' pitch)
+    void* red;          // per strip, kRedN DSum slots of its step-end sums
+    void* red_groups;   // the same per group of strips
+    unsigned* tickets;  // [0] groups, [1 + g] strips of group g that have finished
+    double* stats;
+    double dt;
+    double far_x, far_y;   // -2 H0 (cos, sin): twice the far field's slopes
+    float far_h[2], far_l[2];   // the same as FP32 pairs
+    int nx, ny, pitch, periodic_x, periodic_y;
+    int thermal_dir[4], mag_dir[4];
+    int solve_potential;
+    int strips;         // strips of the case (batch launches)
+    int pad_;
 };
 
 // One block's work: the tile at (x0, y0) of a case; slot numbers the case's
@@ -154,41 +193,6 @@ __device__ __forceinline__ R mix(R Fs, R C, R gs, R gl, R gg) {
     const R liq = gg + C * (gl - gg);
     return liq + Fs * (gs - liq);
 }
-
-// Eq. 8 as above with the two threshold differences H_e - H_es and H_e - H_el formed
-// in precision H and everything after them in R.  Hes_h = C_p,s T_m and L_h = L are
-// given in H.  Used with H = R (the interface enthalpy in the face fluxes) and with
-// H = R = double (the stored enthalpy in FP64 mode); the mixed-precision stored
-// enthalpy, an FP32 pair, goes through invert_hp.
-template <class R, class H>
-__device__ __forceinline__ void invert_h(const PhysT<R>& Q, H Hes_h, H L_h, H He, R C, R& T, R& Fl,
-                                         R* He_r = nullptr) {
-    const R cpL = Q.cp_g + C * (Q.cp_l - Q.cp_g);
-    const bool tm0 = Q.T_m == R(0);   // then H_es = 0 and H_el = L
-    const H Hel = tm0 ? L_h : L_h + H(cpL * Q.T_m);
-    const R ds = tm0 ? R(He) : R(He - Hes_h), dl = R(He - Hel);
-    if (He_r) *He_r = tm0 ? ds : ds + R(Hes_h);   // H_e in R for the reconstruction
-    if (C < R(0.5)) {
-        Fl = R(1);
-        T = Q.T_m + fdiv(dl, cpL);
-    } else if (ds < R(0)) {
-        Fl = R(0);
-        T = Q.T_m + fdiv(ds, Q.cp_s);
-    } else if (dl <= R(0)) {
-        Fl = fdiv(ds, ds - dl);
-        T = Q.T_m;
-    } else {
-        Fl = R(1);
-        T = Q.T_m + fdiv(dl, cpL);
-    }
-}
-
-template <class R>
-__device__ __forceinline__ const PhysT<R>& phys_of(const DevCase* dc);
-template <>
-__device__ __forceinline__ const PhysT<float>& phys_of<float>(const DevCase* dc) { return dc->qf; }
-template <>
-__device__ __forceinline__ const PhysT<double>& phys_of<double>(const DevCase* dc) { return dc->qd; }
 
 // ---- FP64-accurate arithmetic on FP32 pairs (hi + lo, |lo| <= ulp(hi)/2) ---------
 // Error-free transformations: two_sum (Knuth), two_prod (FMA).  Explicit round-to-
@@ -334,42 +338,6 @@ __device__ __forceinline__ void he_set(void* base, size_t k, double v) {
         float2 h;
         pair_from(v, h.x, h.y);
         static_cast<float2*>(base)[k] = h;
-    }
-}
-
-// Eq. 8 (as invert_h) on an FP32-pair enthalpy.  Each threshold difference is formed
-// from the parts, (hi - t_hi) + (lo - t_lo): the high parts of two nearby values
-// subtract exactly, so the difference is within an FP32 rounding of the FP64 one,
-// and no FP64 instruction is needed.
-__device__ __forceinline__ void invert_hp(const PhysT<float>& Q, float2 He, float C, float& T, float& Fl,
-                                          float* He_r = nullptr) {
-    const float cpL = Q.cp_g + C * (Q.cp_l - Q.cp_g);
-    float ds, dl;
-    if (Q.T_m == 0.0f) {   // H_es = 0 and H_el = L
-        ds = __fadd_rn(He.x, He.y);
-        dl = __fadd_rn(__fsub_rn(He.x, Q.L_hi), __fsub_rn(He.y, Q.L_lo));
-        if (He_r) *He_r = ds;
-    } else {
-        float2 Hel;
-        Hel.x = Q.L_hi;
-        Hel.y = Q.L_lo;
-        Hel = pair_add_f(Hel, cpL * Q.T_m);
-        ds = __fadd_rn(__fsub_rn(He.x, Q.Hes_hi), __fsub_rn(He.y, Q.Hes_lo));
-        dl = __fadd_rn(__fsub_rn(He.x, Hel.x), __fsub_rn(He.y, Hel.y));
-        if (He_r) *He_r = ds + Q.Hes_hi;
-    }
-    if (C < 0.5f) {
-        Fl = 1.0f;
-        T = Q.T_m + fdiv(dl, cpL);
-    } else if (ds < 0.0f) {
-        Fl = 0.0f;
-        T = Q.T_m + fdiv(ds, Q.cp_s);
-    } else if (dl <= 0.0f) {
-        Fl = fdiv(ds, ds - dl);
-        T = Q.T_m;
-    } else {
-        Fl = 1.0f;
-        T = Q.T_m + fdiv(dl, cpL);
     }
 }
 

@@ -8,14 +8,19 @@
 
 namespace lbfs {
 
-// stage kernel (lbfs_stage.cu); prec 0 = FP64, 1 = mixed
+// stage kernel (lbfs_stage.cu); prec 0 = FP64, 1 = mixed.  A strip is kStripW columns by
+// `rows` rows of one case, advanced by one warp (a block of its own).
+constexpr int kStripW = 26;
 int stage_tile_shapes();
-int stage_tile_w(int prec, int tile);
-int stage_tile_h(int prec, int tile);
+// rows of a strip for shape id `tile` (0: chosen from the strip-rows of all cases together)
+int stage_rows(int prec, int tile, long long row_warps, int sm_count);
+constexpr int kStageMinRows = 1, kStageGroup = 64;   // lowest strips; strips summed together at the step end
 // half: every case streams half a cell (dts = 1/2), which selects the reconstruction
-// without normal slopes at the upwind points
-cudaError_t launch_stage(int prec, int tile, int half, const DevCase* cases, const TileRef* tiles,
-                         int ntiles, int stage, cudaStream_t st);
+// without normal slopes at the upwind points.  one: the context's only case (host copy), or
+// NULL for a batch, whose strips come from `tiles` and whose cases from `cases`.
+template <class R>
+cudaError_t launch_stage(int half, const StageCase<R>* one, const StageCase<R>* cases, const TileRef* tiles, int ntiles,
+                         int rows, int stage, cudaStream_t st);
 
 // potential multigrid (lbfs_potential.cu).  The fine-level cell kernels (residual,
 // correction) take 32 x 32 tiles.  first: the step's first residual (every case);
@@ -67,7 +72,5 @@ cudaError_t launch_stats_init(int prec, const DevCase* dcase, int nx, int ny, cu
 // {H_m, U_max, Pe, Fo, Q_wall}; two launches.
 cudaError_t launch_diagnostics(int prec, const DevCase* dcase, int nx, double R0, double* cols,
                                double* out5, cudaStream_t st);
-cudaError_t launch_step_finalize(int prec, const DevCase* cases, const int* case_ids, int ncases,
-                                 cudaStream_t st);
 
 }  // namespace lbfs

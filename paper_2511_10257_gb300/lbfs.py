@@ -76,10 +76,10 @@ class CaseDiag(ct.Structure):
 EXPORTS = ("lbfs_create", "lbfs_set_case", "lbfs_set_fields", "lbfs_step", "lbfs_fields",
            "lbfs_diagnostics", "lbfs_potential_pseudo_time", "lbfs_last_launch_count", "lbfs_timing", "lbfs_timing_read", "lbfs_autotune",
            "lbfs_destroy", "lbfs_last_error")
-TILE_SHAPES = [(32, 8), (32, 16), (64, 8), (16, 16), (64, 4), (16, 16), (32, 8), (16, 16), (32, 8), (16, 16),
-               (32, 8), (16, 15), (32, 7)]
-TILE_NAMES = ["32x8", "32x16", "64x8", "16x16", "64x4", "16x16/3", "32x8/3", "16x16/4", "32x8/4", "16x16/4t",
-              "32x8/4t", "16x15/4t", "32x7/4t"]
+# strip shapes of the stage kernel: columns x rows of one warp (0 rows: chosen by the library)
+TILE_SHAPES = [(26, 0), (26, 128), (26, 96), (26, 64), (26, 48), (26, 32), (26, 24), (26, 16), (26, 12), (26, 8), (26, 4),
+               (26, 2), (26, 1)]
+TILE_NAMES = ["auto"] + [f"{w}x{h}" for w, h in TILE_SHAPES[1:]]
 TIMING_STAGE, TIMING_POTENTIAL, TIMING_FINALIZE = range(3)
 
 _lib = None
