@@ -15,8 +15,8 @@ using namespace lbfs;
 
 namespace {
 
-constexpr int kCoarsenCells = 256;    // stop coarsening at or below this many cells
-constexpr int kCoarsestMax = 4096;    // largest coarsest level the one-block CG accepts
+constexpr int kCoarsenCells = 4;      // stop coarsening at or below this many cells
+constexpr int kCoarsestMax = 4096;    // largest coarsest level accepted
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -42,16 +42,20 @@ struct lbfs_ctx {
     void* d_stage_cases = nullptr;   // StageCase of every slot, in the context's precision
     TileRef* d_stage_tiles = nullptr;
     int n_stage_tiles = 0;
-    std::vector<TileRef*> d_mg_tiles;
-    std::vector<int> n_mg_tiles;
+    TileRef* d_mg_tiles = nullptr;      // fine-level 32 x 32 tiles (FP64: the extrapolated start)
+    int n_mg_tiles = 0;
+    TileRef* d_res_tiles = nullptr;     // the residual's strips
+    int n_res_tiles = 0, res_rows = 0;
     std::vector<TileRef*> d_ft_tiles;   // fused V-cycle tiles per level
     std::vector<int> n_ft_tiles;
     std::vector<int> ft_small;          // per level: 16 x 8 fused tiles instead of 32 x 16
     int n_active = 0;
-    int* d_pot = nullptr;
     int n_pot = 0;
-    int max_depth = 0;
-    int coarsest_cells = 0;
+    int* d_tail = nullptr;              // cases whose coarse levels run in one kernel
+    int n_tail = 0, tail_cells = 0, tail_small = 0;
+    int* d_coarsest = nullptr;          // the others: their coarsest level
+    int n_coarsest = 0, coarsest_cells = 0;
+    int max_depth = 0;                  // levels with a kernel per leg
     int sm_count = 152;               // multiprocessors of the context's device
     int* d_flag = nullptr;
     int* h_flag = nullptr;
@@ -319,9 +323,17 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         if (s.defined) row_warps += (long long)((s.hd.P.nx + kStripW - 1) / kStripW) * s.hd.P.ny;
     const int TX = kStripW, TY = stage_rows(ctx->prec, ctx->tile, row_warps, ctx->sm_count);
     ctx->rows = TY;
-    std::vector<int> pot;
-    int active = 0, depth = 0, coarsest = 0;
+    std::vector<int> pot, tails, others;
+    int active = 0, depth = 0, tail_cells = 0, tail_small = 0, coarsest = 0;
     int half = 1;
+    // The residual's strips: 64 rows, or fewer while all of them run at once (24 warps an SM)
+    long long res_warps = 0;
+    for (const Slot& s : ctx->slots)
+        if (s.defined && s.hd.P.solve_potential)
+            res_warps += (long long)((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * s.hd.P.ny;
+    int res_rows = kResidMinRows;
+    while (res_rows < 64 && res_warps > 24LL * ctx->sm_count * res_rows) res_rows *= 2;
+    std::vector<TileRef> rt;
     for (int c = 0; c < (int)ctx->slots.size(); ++c) {
         Slot& s = ctx->slots[c];
         if (!s.defined) continue;
@@ -333,6 +345,12 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             if (cudaMemcpy(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb, cudaMemcpyHostToDevice) != cudaSuccess)
                 return fail(ctx, LBFS_ECUDA, "case table update failed");
         }
+        const int res = ((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * ((s.hd.P.ny + res_rows - 1) / res_rows);
+        if (res != s.hd.mg_strips) {
+            s.hd.mg_strips = res;
+            if (cudaMemcpy(ctx->d_cases + c, &s.hd, sizeof(DevCase), cudaMemcpyHostToDevice) != cudaSuccess)
+                return fail(ctx, LBFS_ECUDA, "case table update failed");
+        }
         ++active;
         if (s.hd.P.dts != 0.5) half = 0;
         int slot = 0;
@@ -340,12 +358,37 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             for (int x = 0; x < s.hd.P.nx; x += TX) st.push_back(TileRef{c, x, y, slot++});
         if (s.hd.P.solve_potential) {
             pot.push_back(c);
-            depth = std::max(depth, s.hd.nlev);
+            depth = std::max(depth, s.hd.tail);
             const MGLevel& lc = s.hd.lev[s.hd.nlev - 1];
-            coarsest = std::max(coarsest, lc.nx * lc.ny);
+            if (lc.nx * lc.ny <= kTailCoarsest) {
+                tails.push_back(c);
+                int cells = 0;
+                int warp_cells = 0;
+                for (int L = s.hd.tail; L < s.hd.nlev; ++L) {
+                    const int n = s.hd.lev[L].nx * s.hd.lev[L].ny;
+                    cells += n;
+                    if (n <= kWarpCells || L == s.hd.nlev - 1) warp_cells += n;
+                }
+                tail_cells = std::max(tail_cells, cells);
+                tail_small = std::max(tail_small, warp_cells);
+            } else {
+                others.push_back(c);
+                coarsest = std::max(coarsest, lc.nx * lc.ny);
+            }
+            slot = 0;
+            for (int y = 0; y < s.hd.P.ny; y += res_rows)
+                for (int x = 0; x < s.hd.P.nx; x += kResidStripW) rt.push_back(TileRef{c, x, y, slot++});
         }
     }
-    std::vector<std::vector<TileRef>> mg(depth), ft(depth);
+    std::vector<TileRef> mg;
+    std::vector<std::vector<TileRef>> ft(depth);
+    if (ctx->prec == 0)
+        for (int c : pot) {
+            const CaseParams& P = ctx->slots[c].hd.P;
+            int slot = 0;
+            for (int y = 0; y < P.ny; y += kMgTY)
+                for (int x = 0; x < P.nx; x += kMgTX) mg.push_back(TileRef{c, x, y, slot++});
+        }
     // A level takes 16 x 8 fused tiles when its 32 x 16 tiles over all cases would
     // leave most SMs idle (fewer than two a multiprocessor): the legs of a small grid
     // then spread over four times as many SMs, at a larger halo share.
@@ -354,7 +397,7 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         long long big = 0;
         for (int c : pot) {
             const Slot& s = ctx->slots[c];
-            if (s.hd.nlev - 1 > L)
+            if (s.hd.tail > L)
                 big += (long long)((s.hd.lev[L].nx + kFusedTX - 1) / kFusedTX) *
                        ((s.hd.lev[L].ny + kFusedTY - 1) / kFusedTY);
         }
@@ -364,15 +407,10 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         const int fx = small[L] ? kFusedSmallTX : kFusedTX, fy = small[L] ? kFusedSmallTY : kFusedTY;
         for (int c : pot) {
             const Slot& s = ctx->slots[c];
-            if (s.hd.nlev <= L) continue;
+            if (s.hd.tail <= L) continue;
             int slot = 0;
-            for (int y = 0; y < s.hd.lev[L].ny; y += kMgTY)
-                for (int x = 0; x < s.hd.lev[L].nx; x += kMgTX) mg[L].push_back(TileRef{c, x, y, slot++});
-            if (s.hd.nlev - 1 > L) {
-                slot = 0;
-                for (int y = 0; y < s.hd.lev[L].ny; y += fy)
-                    for (int x = 0; x < s.hd.lev[L].nx; x += fx) ft[L].push_back(TileRef{c, x, y, slot++});
-            }
+            for (int y = 0; y < s.hd.lev[L].ny; y += fy)
+                for (int x = 0; x < s.hd.lev[L].nx; x += fx) ft[L].push_back(TileRef{c, x, y, slot++});
         }
     }
     ctx->ft_small = small;
@@ -385,21 +423,26 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
     if (!upload((void**)&ctx->d_stage_tiles, st.data(), st.size() * sizeof(TileRef)) ||
-    !upload((void**)&ctx->d_pot, pot.data(), pot.size() * sizeof(int)))
+        !upload((void**)&ctx->d_mg_tiles, mg.data(), mg.size() * sizeof(TileRef)) ||
+        !upload((void**)&ctx->d_res_tiles, rt.data(), rt.size() * sizeof(TileRef)) ||
+        !upload((void**)&ctx->d_tail, tails.data(), tails.size() * sizeof(int)) ||
+        !upload((void**)&ctx->d_coarsest, others.data(), others.size() * sizeof(int)))
         return fail(ctx, LBFS_ENOMEM, "tile list upload failed");
-    for (auto* p : ctx->d_mg_tiles) dfree(ctx, p);
     for (auto* p : ctx->d_ft_tiles) dfree(ctx, p);
-    ctx->d_mg_tiles.assign(depth, nullptr);
-    ctx->n_mg_tiles.assign(depth, 0);
     ctx->d_ft_tiles.assign(depth, nullptr);
     ctx->n_ft_tiles.assign(depth, 0);
     for (int L = 0; L < depth; ++L) {
-        if (!upload((void**)&ctx->d_mg_tiles[L], mg[L].data(), mg[L].size() * sizeof(TileRef)) ||
-            !upload((void**)&ctx->d_ft_tiles[L], ft[L].data(), ft[L].size() * sizeof(TileRef)))
+        if (!upload((void**)&ctx->d_ft_tiles[L], ft[L].data(), ft[L].size() * sizeof(TileRef)))
             return fail(ctx, LBFS_ENOMEM, "multigrid tile list upload failed");
-        ctx->n_mg_tiles[L] = (int)mg[L].size();
         ctx->n_ft_tiles[L] = (int)ft[L].size();
     }
+    ctx->n_mg_tiles = (int)mg.size();
+    ctx->n_res_tiles = (int)rt.size();
+    ctx->res_rows = res_rows;
+    ctx->n_tail = (int)tails.size();
+    ctx->tail_cells = tail_cells;
+    ctx->tail_small = tail_small;
+    ctx->n_coarsest = (int)others.size();
     ctx->n_stage_tiles = (int)st.size();
     ctx->n_active = active;
     ctx->n_pot = (int)pot.size();
@@ -418,19 +461,28 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             return fail(ctx, LBFS_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// One V-cycle on the correction equation A e = r of every solving case: a fused
-// pre-smooth + restriction kernel per level on the way down, the one-block CG on each
-// case's coarsest level, a fused prolongation + post-smooth kernel per level up.
+// One V-cycle on the correction equation A e = r of every solving case, ending with phi += e:
+// a fused pre-smooth + restriction kernel per level on the way down, the coarse levels in one
+// kernel per case (or conjugate gradients on a coarsest level too large for it), a fused
+// prolongation + post-smooth kernel per level up.
 lbfs_status vcycle(lbfs_ctx* ctx) {
     const int p = ctx->prec;
     cudaStream_t s = ctx->stream;
     const int D = ctx->max_depth;
-    for (int L = 0; L + 1 < D; ++L)
+    for (int L = 0; L < D; ++L)
         LK(launch_mg_vdown(p, ctx->d_cases, ctx->d_ft_tiles[L], ctx->n_ft_tiles[L], L, ctx->ft_small[L], s));
-    LK(launch_mg_coarsest(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->coarsest_cells, s));
-    for (int L = D - 2; L >= 0; --L)
+    if (ctx->n_tail > 0) LK(launch_mg_tail(p, ctx->d_cases, ctx->d_tail, ctx->n_tail, ctx->tail_cells, ctx->tail_small, s));
+    if (ctx->n_coarsest > 0) LK(launch_mg_coarsest(ctx->d_cases, ctx->d_coarsest, ctx->n_coarsest, ctx->coarsest_cells, s));
+    for (int L = D - 1; L >= 0; --L)
         LK(launch_mg_vup(p, ctx->d_cases, ctx->d_ft_tiles[L], ctx->n_ft_tiles[L], L, ctx->ft_small[L], s));
     return LBFS_OK;
+}
+
+// the residual of the master potential and each case's check
+cudaError_t check_residual(lbfs_ctx* ctx, int first, int kmax, int* not_done, unsigned* ticket,
+                           cudaGraphConditionalHandle cond, int set_cond) {
+    PotCheck ck{first, ctx->mg_tol, kmax, not_done, ticket, ctx->n_pot, cond, set_cond};
+    return launch_mg_residual(ctx->prec, ctx->d_cases, ctx->d_res_tiles, ctx->n_res_tiles, ctx->res_rows, ck, ctx->stream);
 }
 
 // The warm potential solve, recorded into the graph being captured on ctx->stream:
@@ -451,12 +503,8 @@ lbfs_status capture_warm_potential(lbfs_ctx* ctx) {
     if (cs != cudaStreamCaptureStatusActive || !g) return fail(ctx, LBFS_ECUDA, "potential capture is not active");
     cudaGraphConditionalHandle h;
     CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
-    if (p == 0) {
-        LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], ctx->d_pot, ctx->n_pot, s));
-        ++ctx->launches;
-    }
-    LK(launch_mg_residual64(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], 1, s));
-    LK(launch_mg_finalize(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->mg_tol, 1, K, nd, ticket, h, 1, s));
+    if (p == 0) LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
+    LK(check_residual(ctx, 1, K, nd, ticket, h, 1));
     const cudaGraphNode_t* deps = nullptr;
     size_t ndeps = 0;
     CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &ndeps));
@@ -478,12 +526,8 @@ lbfs_status capture_warm_potential(lbfs_ctx* ctx) {
     const int64_t l0 = ctx->launches;
     lbfs_status r = vcycle(ctx);
     if (r == LBFS_OK) {
-        cudaStream_t b = ctx->body_stream;
-        cudaError_t e = launch_mg_correct(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], b);
-        if (e == cudaSuccess) e = launch_mg_residual64(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], 0, b);
-        if (e == cudaSuccess)
-            e = launch_mg_finalize(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->mg_tol, 0, K, nd, ticket, h, 1, b);
-        ctx->launches += 3;
+        const cudaError_t e = check_residual(ctx, 0, K, nd, ticket, h, 1);
+        ++ctx->launches;
         if (e != cudaSuccess) r = fail(ctx, LBFS_ECUDA, std::string("cycle body: ") + cudaGetErrorString(e));
     }
     ctx->cycle_launches = ctx->launches - l0;
@@ -537,19 +581,12 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
         // the same cycles as plain launches; each kernel returns at once for a converged case
         const int K = ctx->mg_warm_cycles;
         int* nd = ctx->d_flag + 1;
-        if (p == 0) {
-            LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], ctx->d_pot, ctx->n_pot,
-                                     s));
-            ++ctx->launches;
-        }
-        LK(launch_mg_residual64(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], 1, s));
-        LK(launch_mg_finalize(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->mg_tol, 1, K, nd, nullptr, 0, 0, s));
+        if (p == 0) LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
+        LK(check_residual(ctx, 1, K, nd, nullptr, 0, 0));
         for (int c = 0; c < K; ++c) {
             lbfs_status r = vcycle(ctx);
             if (r != LBFS_OK) return r;
-            LK(launch_mg_correct(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], s));
-            LK(launch_mg_residual64(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], 0, s));
-            LK(launch_mg_finalize(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->mg_tol, 0, K, nd, nullptr, 0, 0, s));
+            LK(check_residual(ctx, 0, K, nd, nullptr, 0, 0));
         }
         CK(cudaMemsetAsync(nd, 0, sizeof(int), s));
         return LBFS_OK;
@@ -561,14 +598,12 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
             if (r != LBFS_OK) return r;
         }
         CK(cudaGraphLaunch(ctx->pot_exec, s));
-        ctx->launches += p == 0 ? 4 : 2;   // (FP64: the extrapolated start) residual, check
+        ctx->launches += p == 0 ? 2 : 1;   // (FP64: the extrapolated start) residual with its check
         return LBFS_OK;
     }
     for (int it = 0;; ++it) {
-        LK(launch_mg_residual64(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], it == 0, s));
         CK(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s));
-        LK(launch_mg_finalize(p, ctx->d_cases, ctx->d_pot, ctx->n_pot, ctx->mg_tol, it == 0, 1 << 30, ctx->d_flag,
-                              nullptr, 0, 0, s));
+        LK(check_residual(ctx, it == 0, 1 << 30, ctx->d_flag, nullptr, 0, 0));
         CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (*ctx->h_flag == 0) break;
@@ -578,7 +613,6 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
         }
         lbfs_status r = vcycle(ctx);
         if (r != LBFS_OK) return r;
-        LK(launch_mg_correct(p, ctx->d_cases, ctx->d_mg_tiles[0], ctx->n_mg_tiles[0], s));
     }
     // the warm steps that follow extrapolate only once they have stored a potential
     for (size_t c = 0; c < ctx->slots.size(); ++c)
@@ -695,19 +729,25 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
         }
         ctx->own_stream = true;
     }
-    ctx->d_cases = static_cast<DevCase*>(dalloc(ctx, sizeof(DevCase) * cfg->max_cases));
-    ctx->d_stage_cases = dalloc(ctx, (ctx->prec == 0 ? sizeof(StageCase<double>) : sizeof(StageCase<float>)) * cfg->max_cases);
-    ctx->d_stats = static_cast<double*>(dalloc(ctx, sizeof(double) * kStatN * cfg->max_cases));
-    ctx->d_flag = static_cast<int*>(dalloc(ctx, 256));
-    if (!ctx->d_cases || !ctx->d_stage_cases || !ctx->d_stats || !ctx->d_flag ||
+    // the context's tables in one allocation
+    const size_t cases_b = align_up(sizeof(DevCase) * cfg->max_cases, 256);
+    const size_t stage_b =
+        align_up((ctx->prec == 0 ? sizeof(StageCase<double>) : sizeof(StageCase<float>)) * cfg->max_cases, 256);
+    const size_t stats_b = align_up(sizeof(double) * kStatN * cfg->max_cases, 256);
+    ctx->d_cases = static_cast<DevCase*>(dalloc(ctx, cases_b + stage_b + stats_b + 256));
+    if (ctx->d_cases) {
+        char* base = reinterpret_cast<char*>(ctx->d_cases);
+        ctx->d_stage_cases = base + cases_b;
+        ctx->d_stats = reinterpret_cast<double*>(base + cases_b + stage_b);
+        ctx->d_flag = reinterpret_cast<int*>(base + cases_b + stage_b + stats_b);
+    }
+    if (!ctx->d_cases ||
         cudaMallocHost(&ctx->h_flag, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_stats, sizeof(double) * kStatN * cfg->max_cases) != cudaSuccess) {
         lbfs_destroy(ctx);
         return LBFS_ENOMEM;
     }
-    cudaMemset(ctx->d_cases, 0, sizeof(DevCase) * cfg->max_cases);
-    cudaMemset(ctx->d_flag, 0, 256);   // [0] host-checked votes, [1] device votes, [2] ticket
-    cudaMemset(ctx->d_stats, 0, sizeof(double) * kStatN * cfg->max_cases);
+    cudaMemset(ctx->d_cases, 0, cases_b + stage_b + stats_b + 256);   // d_flag: [0] host-checked votes, [1] device votes, [2] ticket
     if (cudaDeviceSynchronize() != cudaSuccess) {
         lbfs_destroy(ctx);
         return LBFS_ECUDA;
@@ -758,7 +798,16 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     hd.nlev = nlev;
     // partial-sum slots for the lowest strips
     const int red_cap = ((P.nx + kStripW - 1) / kStripW) * ((P.ny + kStageMinRows - 1) / kStageMinRows);
-    hd.mg_tiles = ((P.nx + kMgTX - 1) / kMgTX) * ((P.ny + kMgTY - 1) / kMgTY);
+    const int res_cap = ((P.nx + kResidStripW - 1) / kResidStripW) * ((P.ny + kResidMinRows - 1) / kResidMinRows);
+    const int res_groups = (res_cap + kStageGroup - 1) / kStageGroup;
+    // the levels that run in one kernel per case
+    hd.tail = nlev - 1;
+    if (nx * ny <= kTailCoarsest)
+        while (hd.tail > 0 && hd.lev[hd.tail - 1].nx * hd.lev[hd.tail - 1].ny <= kTailCells) --hd.tail;
+    hd.far_h[0] = (float)(-P.H0 * P.cos_t);
+    hd.far_l[0] = (float)(-P.H0 * P.cos_t - (double)hd.far_h[0]);
+    hd.far_h[1] = (float)(-P.H0 * P.sin_t);
+    hd.far_l[1] = (float)(-P.H0 * P.sin_t - (double)hd.far_h[1]);
     // one device block per case
     const size_t rs = ctx->prec == 0 ? sizeof(double) : sizeof(float);
     const size_t cells = (size_t)P.pitch * P.ny;
@@ -784,17 +833,19 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     for (int L = 0; L < nlev; ++L) {
         hd.lev[L].pitch = (int)align_up((size_t)hd.lev[L].nx, 32);
         const size_t lc = (size_t)hd.lev[L].pitch * hd.lev[L].ny;
-        add(&hd.lev[L].mu, lc * rs);
-        add(&hd.lev[L].e, lc * rs);
-        add(&hd.lev[L].r, lc * rs);
+        add(&hd.lev[L].mu, lc * (L == 0 ? rs : sizeof(float)));
+        add(&hd.lev[L].e, lc * sizeof(float));
+        add(&hd.lev[L].r, lc * (L == 0 ? rs : sizeof(float)));
     }
     const int red_groups = (red_cap + kStageGroup - 1) / kStageGroup;
     add((void**)&hd.red, (size_t)red_cap * kRedN * sizeof(double));
     add((void**)&hd.red_groups, (size_t)red_groups * kRedN * sizeof(double));
     add((void**)&hd.red_tickets, (size_t)(1 + red_groups) * sizeof(unsigned));
-    add((void**)&hd.mg_red, (size_t)hd.mg_tiles * 2 * sizeof(double));
-    add((void**)&hd.chunk, (size_t)kFinChunks * (kRedN + 2) * sizeof(double));
-    add((void**)&hd.tickets, 2 * sizeof(unsigned));
+    add((void**)&hd.mg_red, (size_t)res_cap * 2 * sizeof(double));
+    add((void**)&hd.mg_groups, (size_t)res_groups * 2 * sizeof(double));
+    add((void**)&hd.mg_tickets, (size_t)(1 + res_groups) * sizeof(unsigned));
+    add((void**)&hd.chunk, (size_t)kFinChunks * kRedN * sizeof(double));
+    add((void**)&hd.tickets, sizeof(unsigned));
     Slot& s = ctx->slots[id];
     free_slot(ctx, s);
     drop_graph(ctx);
@@ -1081,14 +1132,13 @@ void lbfs_destroy(lbfs_ctx* ctx) {
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->body_stream) cudaStreamDestroy(ctx->body_stream);
     for (Slot& s : ctx->slots) free_slot(ctx, s);
-    for (auto* p : ctx->d_mg_tiles) dfree(ctx, p);
     for (auto* p : ctx->d_ft_tiles) dfree(ctx, p);
-    dfree(ctx, ctx->d_stage_cases);
+    dfree(ctx, ctx->d_mg_tiles);
+    dfree(ctx, ctx->d_res_tiles);
+    dfree(ctx, ctx->d_tail);
+    dfree(ctx, ctx->d_coarsest);
     dfree(ctx, ctx->d_stage_tiles);
-    dfree(ctx, ctx->d_pot);
     dfree(ctx, ctx->d_cases);
-    dfree(ctx, ctx->d_stats);
-    dfree(ctx, ctx->d_flag);
     dfree(ctx, ctx->d_scratch);
     if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
     if (ctx->h_stats) cudaFreeHost(ctx->h_stats);

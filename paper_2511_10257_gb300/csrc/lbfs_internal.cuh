@@ -17,7 +17,7 @@ constexpr int kStatN = 20;      // per-case device statistics slots
 enum StatSlot {
     ST_SUM_C = 0, ST_SUM_HE, ST_SUM_FL_DROP, ST_N_DROP, ST_Q_L, ST_T, ST_T_FREEZE,
     ST_POT_RESID, ST_POT_CYCLES, ST_NONFINITE, ST_QL_PREV, ST_POT_DONE, ST_B2, ST_STEP,
-    ST_POT_FAIL, ST_POT_RESID_MAX, ST_POT_CYCLES_SUM, ST_STEPS_CALL, ST_EXTRAP, ST_SPARE1
+    ST_POT_FAIL, ST_POT_RESID_MAX, ST_POT_CYCLES_SUM, ST_STEPS_CALL, ST_EXTRAP, ST_SCALE
 };
 
 // Physical and numerical parameters of one case, resolved on the host in FP64.
@@ -75,9 +75,9 @@ struct MGLevel {
     // width (height) relative to the level's other cells, 1 when the level is regular.
     float wlx, wly;
     int ragged;  // wlx < 1 or wly < 1
-    void* mu;   // cell coefficient mu_m (M precision)
-    void* e;    // correction
-    void* r;    // right-hand side / residual
+    void* mu;   // cell coefficient mu_m (FP32; FP64 on the fine level of the FP64 mode)
+    void* e;    // correction (FP32)
+    void* r;    // right-hand side / residual (as mu)
 };
 
 // Everything the kernels need to know about one case.
@@ -97,10 +97,14 @@ struct DevCase {
     void* red;        // stage-strip partial sums, kRedN 8-byte DSum slots per strip
     void* red_groups; // the same per group of strips
     unsigned* red_tickets;
-    void* mg_red;     // potential residual partial sums, 2 DSum slots per fine tile
-    void* chunk;      // kFinChunks x (kRedN + 2) DSum slots: per-chunk sums of the partials
-    unsigned* tickets;  // [0] set-up statistics, [1] residual: chunks done (the last one finalises)
-    int mg_tiles;
+    int tail;         // level from which the V-cycle runs in one kernel (nlev - 1: the coarsest alone)
+    void* mg_red;     // potential residual partial sums, 2 DSum slots per residual strip
+    void* mg_groups;  // the same per group of strips
+    unsigned* mg_tickets;   // [0] groups, [1 + g] strips of group g that have finished
+    int mg_strips;
+    float far_h[2], far_l[2];   // the far field's slopes -H0 (cos, sin) as FP32 pairs
+    void* chunk;      // kFinChunks x kRedN DSum slots: per-chunk sums of the set-up statistics
+    unsigned* tickets;  // set-up statistics: chunks done (the last one finalises)
     double* stats;    // kStatN FP64 slots
 };
 
@@ -255,6 +259,7 @@ struct DSum<double> {
     __device__ __forceinline__ void add(DSum o) { v += o.v; }
     __device__ __forceinline__ void sub(DSum o) { v -= o.v; }
     __device__ __forceinline__ void shfl_add(int o) { v += __shfl_down_sync(0xffffffffu, v, o); }
+    __device__ __forceinline__ void shfl_xor_add(int o) { v += __shfl_xor_sync(0xffffffffu, v, o); }
     __device__ __forceinline__ Slot slot() const { return v; }
     __device__ __forceinline__ double value() const { return v; }
 };
@@ -280,6 +285,12 @@ struct DSum<float> {
         w.y = __shfl_down_sync(0xffffffffu, v.y, o);
         v = pair_add2(v, w);
     }
+    __device__ __forceinline__ void shfl_xor_add(int o) {
+        float2 w;
+        w.x = __shfl_xor_sync(0xffffffffu, v.x, o);
+        w.y = __shfl_xor_sync(0xffffffffu, v.y, o);
+        v = pair_add2(v, w);
+    }
     __device__ __forceinline__ Slot slot() const { return v; }
     __device__ __forceinline__ double value() const { return (double)v.x + (double)v.y; }
 };
@@ -297,6 +308,18 @@ __device__ __forceinline__ DSum<R> block_sum0(DSum<R> v, typename DSum<R>::Slot*
     if (threadIdx.x == 0)
         for (int q = 0; q < (int)((blockDim.x + 31) >> 5); ++q) tot.add(DSum<R>::of(sh[q]));
     return tot;
+}
+
+// whether this warp is the last of n to arrive at the ticket, which it then clears
+__device__ __forceinline__ bool last_of(unsigned* ticket, int n, int lane) {
+    unsigned last = 0;
+    if (lane == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == (unsigned)(n - 1);
+        if (last) *ticket = 0u;
+        __threadfence();
+    }
+    return __shfl_sync(0xffffffffu, last, 0) != 0;
 }
 
 // load that bypasses L1 (data written by other blocks of the same launch)

@@ -22,31 +22,40 @@ template <class R>
 cudaError_t launch_stage(int half, const StageCase<R>* one, const StageCase<R>* cases, const TileRef* tiles, int ntiles,
                          int rows, int stage, cudaStream_t st);
 
-// potential multigrid (lbfs_potential.cu).  The fine-level cell kernels (residual,
-// correction) take 32 x 32 tiles.  first: the step's first residual (every case);
-// later ones skip converged cases.
+// potential multigrid (lbfs_potential.cu).  The extrapolation takes 32 x 32 tiles.
 constexpr int kMgTX = 32, kMgTY = 32;
-cudaError_t launch_mg_residual64(int prec, const DevCase* cases, const TileRef* tiles, int n, int first,
-                                 cudaStream_t st);
-// tol: the convergence test.  first: the step's first check.  A case still above tol
-// gets another cycle (one more vote in not_done) unless it has had kmax, when it is
-// marked as failed.  set_cond: the call runs inside a conditional graph node; the
-// last case to decide (ticket) sets cond to 1 while a case needs another cycle.
+// The residual takes strips of kResidStripW columns by `rows` rows, one warp each, and checks
+// each case once its strips are done.  first: the step's first residual (every case; later ones
+// skip converged cases).  tol: the convergence test.  A case still above tol gets another cycle
+// (one more vote in not_done) unless it has had kmax, when it is marked as failed.  set_cond:
+// the call runs inside a conditional graph node; the last of ncases to decide (ticket) sets cond
+// to 1 while a case needs another cycle.
+constexpr int kResidStripW = 30, kResidMinRows = 2;
+struct PotCheck {
+    int first;
+    double tol;
+    int kmax;
+    int* not_done;
+    unsigned* ticket;
+    int ncases;
+    cudaGraphConditionalHandle cond;
+    int set_cond;
+};
+cudaError_t launch_mg_residual(int prec, const DevCase* cases, const TileRef* tiles, int n, int rows, const PotCheck& ck,
+                               cudaStream_t st);
 // `iters` explicit pseudo-time steps of the paper's magnetic LBFS (Eqs. 12-18) on one
 // case, FP64 arithmetic; tmp holds nx*ny doubles.  2 launches per step.
 cudaError_t launch_pseudo_time(int prec, const DevCase* dcase, int nx, int ny, int iters, double dtau,
                                double* tmp, cudaStream_t st);
-cudaError_t launch_mg_finalize(int prec, const DevCase* cases, const int* case_ids, int ncases, double tol, int first,
-                               int kmax, int* not_done, unsigned* ticket, cudaGraphConditionalHandle cond,
-                               int set_cond, cudaStream_t st);
-cudaError_t launch_mg_coarsest(int prec, const DevCase* cases, const int* case_ids, int ncases,
-                               int max_cells, cudaStream_t st);
-// FP64 only: the linearly extrapolated warm start of the potential (two launches)
-cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, const int* ids, int ncases,
-                                  cudaStream_t st);
-cudaError_t launch_mg_correct(int prec, const DevCase* cases, const TileRef* tiles, int n,
-                              cudaStream_t st);
-size_t mg_coarsest_smem(int prec, int max_cells);
+// The V-cycle's levels from DevCase::tail down, one block per case.  A case takes it when its
+// coarsest level holds at most kTailCoarsest cells, from the first level of at most kTailCells.
+constexpr int kTailCells = 2048, kTailCoarsest = 1024, kWarpCells = 32, kPassCells = 256;   // (kWarpCells: levels of one warp)
+cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* case_ids, int ncases, int max_cells, int max_small,
+                           cudaStream_t st);
+// the coarsest level of the other cases
+cudaError_t launch_mg_coarsest(const DevCase* cases, const int* case_ids, int ncases, int max_cells, cudaStream_t st);
+// FP64 only: the linearly extrapolated warm start of the potential
+cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, cudaStream_t st);
 // fused V-cycle legs over 32 x 16 tiles of one level (kFusedTX x kFusedTY), or over
 // 16 x 8 tiles (small != 0) on a level whose 32 x 16 tiles would not fill the GPU
 constexpr int kFusedTX = 32, kFusedTY = 16;

@@ -1,9 +1,13 @@
 // lbfs_potential.cu -- the magnetic scalar potential, div(mu_m grad phi) = 0 (Eq. 4),
 // on the cell-centred five-point stencil with the arithmetic-mean face coefficient:
 // the steady state of the paper's magnetic LBFS (Eqs. 12-18) at a half-cell streaming
-// step.  Solved by residual refinement: the residual r = b - A phi is formed in FP64
-// against the FP64 master potential, the correction A e = r by one multigrid V-cycle
-// in the working precision M (FP32 in mixed mode), then phi += e.
+// step.  Solved by residual refinement: the residual r = b - A phi is formed in FP64, or in
+// FP32 pairs in mixed precision, against the master potential, the correction A e = r by one
+// multigrid V-cycle in FP32, then phi += e.  The residual alone decides when the potential is
+// converged, so the precision of the correction enters only through the number of cycles
+// (the contraction of 0.10-0.16 a cycle is far above FP32 rounding); in the FP64 mode the
+// residual is scaled by a power of two on its way into the correction, so that FP32's range
+// does not matter either.
 //
 // Operator (per level, homogeneous walls for the correction):
 //   (A x)_c = sum_nb mu_f (x_c - x_nb) + sum_Dirichlet-walls 2 mu_c x_c,
@@ -16,6 +20,8 @@
 // carry the true face length over centre distance, and the prolongation interpolates
 // between the true centres, so every grid size keeps the contraction of the even
 // ones.
+#include <type_traits>
+
 #include "lbfs_kernels.h"
 
 namespace lbfs {
@@ -128,154 +134,131 @@ __device__ __forceinline__ M apply_A(const CaseParams& P, const MGLevel& lv, con
     return acc;
 }
 
-// FP64-accurate residual of the master potential on the fine level and per-tile
-// partial sums of |r|^2 and |b|^2.
-//   r = b - A phi = -[sum_nb mu_f (phi_c - phi_nb) + sum_Dirichlet 2 mu_c (phi_c - phi_w)]
-// FP64 mode: in FP64.  Mixed mode: the master potential is the FP32 pair phi + phi_lo
-// and the differences, products and sums are error-free pair operations on the FP32
-// pipes (about 2^-48 relative), because FP64 issue is scarce on GB300; only the norms
-// are accumulated in FP64.
-template <class M>
-__device__ __forceinline__ double residual_cell(const DevCase* dc, const CaseParams& P, const MGLevel& lv,
-                                                int i, int j, double& b_out);
+// ---- residual and check ------------------------------------------------------------
+// r = b - A phi written with face terms: T = mu_f (phi_c - phi_nb) on the lower/left face of
+// a cell serves the cell on either side, and a Dirichlet wall is a face to the wall value with
+// coefficient 2 mu_c (an insulating wall one with coefficient 0), so
+//   r_c = T(right) - T(left) + T(top) - T(bottom).
+// FP64 mode: in FP64.  Mixed mode: the master potential is the FP32 pair phi + phi_lo, and the
+// differences, products and sums are error-free pair operations on the FP32 pipes (about
+// 2^-48 relative; GB300's FP64 issue is scarce), both faces of a cell as the two lanes of the
+// packed instructions.
 
+// a pair of values per axis: (h, l) each for the left face (x) and the lower face (y)
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    s = __fadd2_rn(a, b);
+    const float2 bb = __ffma2_rn(a, m1, s);
+    e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m1, s), m1, a), __ffma2_rn(bb, m1, b));
+}
+
+template <class M>
+struct FaceTerm;
 template <>
-__device__ __forceinline__ double residual_cell<double>(const DevCase* dc, const CaseParams& P,
-                                                        const MGLevel& lv, int i, int j, double& b_out) {
-    const double* mu = static_cast<const double*>(lv.mu);
-    const double* ph = dc->phi64;
-    const size_t k = (size_t)j * lv.pitch + i;
-    const double mc = mu[k], pc = ph[k];
-    double diag = 0.0, off = 0.0, b = 0.0;
-    for (int w = 0; w < 4; ++w) {
-        int ii, jj;
-        if (neighbour(P, lv.nx, lv.ny, i, j, w, ii, jj)) {
-            const size_t kn = (size_t)jj * lv.pitch + ii;
-            const double mf = 0.5 * (mc + mu[kn]);
-            diag += mf;
-            off += mf * ph[kn];
-        } else if (P.mag_dir[w]) {
-            const double wx = w == 0 ? 0.0 : (w == 1 ? (double)lv.nx : i + 0.5);
-            const double wy = w == 2 ? 0.0 : (w == 3 ? (double)lv.ny : j + 0.5);
-            const double pw = -P.H0 * (wx * P.cos_t + wy * P.sin_t);
-            diag += 2.0 * mc;
-            b += 2.0 * mc * pw;
-        }
-    }
-    b_out = b;
-    return b - (diag * pc - off);
-}
+struct FaceTerm<double> {
+    double x, y;   // T of the left and of the lower face
+};
+template <>
+struct FaceTerm<float> {
+    float2 h, l;   // T = h + l; lane x the left face, lane y the lower face
+};
 
-// mixed precision: r rounded to FP32 (it feeds the FP32 correction solve); b and its
-// FP64 wall terms only at cells next to a Dirichlet wall (has_b)
-__device__ __forceinline__ float residual_cell_f(const DevCase* dc, const CaseParams& P, const MGLevel& lv,
-                                                 int i, int j, double& b_out, bool& has_b) {
-    const float* mu = static_cast<const float*>(lv.mu);
-    const float* hi = static_cast<const float*>(dc->phi);
-    const float* lo = dc->phi_lo;
-    // 32-bit cell indices: a level holds fewer than 2^31 cells (checked at set-up)
-    const unsigned pitch = (unsigned)lv.pitch;
-    const unsigned k = (unsigned)j * pitch + (unsigned)i;
-    const float mc = mu[k], hc = hi[k], lc = lo[k];
-    float ah = 0.f, al = 0.f;   // A phi as a pair
-    double b = 0.0;
-    has_b = false;
-    // (phi_c - phi_n) c added to A phi, error-free in pairs
-    auto term = [&](float c, float nh, float nl) {
-        float dh, de, p, pe;
-        two_sum(hc, -nh, dh, de);
-        const float dl = __fadd_rn(de, __fsub_rn(lc, nl));
-        two_prod(c, dh, p, pe);
-        pe = __fmaf_rn(c, dl, pe);
-        pair_add(ah, al, p, pe);
-    };
-    if (i > 0 && i < lv.nx - 1 && j > 0 && j < lv.ny - 1) {
-        // interior cell: four neighbour cells, no wall term (no FP64 instruction)
-        const unsigned kw[4] = {k - 1, k + 1, k - pitch, k + pitch};
-#pragma unroll
-        for (int w = 0; w < 4; ++w) term(0.5f * (mc + mu[kw[w]]), hi[kw[w]], lo[kw[w]]);
-        b_out = 0.0;
-        return -__fadd_rn(ah, al);
-    }
-    for (int w = 0; w < 4; ++w) {
-        int ii, jj;
-        float c, nh, nl;
-        if (neighbour(P, lv.nx, lv.ny, i, j, w, ii, jj)) {
-            const unsigned kn = (unsigned)jj * pitch + (unsigned)ii;
-            c = 0.5f * (mc + mu[kn]);
-            nh = hi[kn];
-            nl = lo[kn];
-        } else if (P.mag_dir[w]) {
-            const double wx = w == 0 ? 0.0 : (w == 1 ? (double)lv.nx : i + 0.5);
-            const double wy = w == 2 ? 0.0 : (w == 3 ? (double)lv.ny : j + 0.5);
-            const double pw = -P.H0 * (wx * P.cos_t + wy * P.sin_t);
-            c = 2.f * mc;
-            pair_from(pw, nh, nl);
-            b += (double)c * pw;
-            has_b = true;
-        } else {
-            continue;
-        }
-        term(c, nh, nl);
-    }
-    b_out = b;
-    return -__fadd_rn(ah, al);
-}
-
-// One block per 32 x 32 tile of the fine level, each thread four rows of a column
-// (rows interleaved so that a warp covers one row); the tile's partial norms are
-// reduced once.  first: the step's first residual, which every case computes; later
-// residuals skip the cases whose solve has converged.
 template <class M>
-__global__ void __launch_bounds__(kNT) k_residual64(const DevCase* __restrict__ cases,
-                                                    const TileRef* __restrict__ tiles, int first) {
-    using Slot = typename DSum<M>::Slot;
-    __shared__ Slot sh[32];
-    const TileRef tr = tiles[blockIdx.x];
-    const DevCase* dc = cases + tr.case_id;
-    if (!first && pot_done(dc)) return;
+struct PotCell;   // one cell's master potential and coefficient
+template <>
+struct PotCell<double> {
+    double v, mu;
+};
+template <>
+struct PotCell<float> {
+    float v, lo, mu;
+};
+
+// Far field -H0 (x cos a + y sin a) at a wall face.  ix, iy: the face's whole coordinates;
+// half: the half cell of its centre belongs to x (0) or y (1).  In mixed precision an FP32
+// pair, formed without FP64 instructions while the coordinates are exact in FP32.
+__device__ __forceinline__ double far_field(const DevCase* dc, int ix, int iy, int half) {
     const CaseParams& P = dc->P;
-    const MGLevel lv = dc->lev[0];
-    DSum<M> r2 = DSum<M>::zero(), b2 = DSum<M>::zero();
-    const int i = tr.x0 + threadIdx.x % kMgTX;
-#pragma unroll
-    for (int q = 0; q < kRowsPT; ++q) {
-        const int j = tr.y0 + threadIdx.x / kMgTX + q * (kNT / kMgTX);
-        if (i < lv.nx && j < lv.ny) {
-            const unsigned k = (unsigned)j * (unsigned)lv.pitch + (unsigned)i;
-            double b;
-            if constexpr (sizeof(M) == 8) {
-                const double r = residual_cell<double>(dc, P, lv, i, j, b);
-                static_cast<double*>(lv.r)[k] = r;
-                r2.add(r * r);
-                b2.add(b * b);
-            } else {
-                bool has_b;
-                const float r = residual_cell_f(dc, P, lv, i, j, b, has_b);
-                static_cast<float*>(lv.r)[k] = r;
-                r2.add(r * r);
-                if (has_b) {
-                    float2 bb;
-                    pair_from(b * b, bb.x, bb.y);
-                    b2.add(bb);
-                }
-            }
-        }
+    return -P.H0 * ((ix + (half == 0 ? 0.5 : 0.0)) * P.cos_t + (iy + (half == 1 ? 0.5 : 0.0)) * P.sin_t);
+}
+__device__ __forceinline__ float2 far_pair(const DevCase* dc, int ix, int iy, int half) {
+    float2 r;
+    if (max(dc->P.nx, dc->P.ny) < (1 << 22)) {
+        const float wx = (float)ix + (half == 0 ? 0.5f : 0.0f), wy = (float)iy + (half == 1 ? 0.5f : 0.0f);
+        float p, e, q, f, s, t;
+        two_prod(dc->far_h[0], wx, p, e);
+        two_prod(dc->far_h[1], wy, q, f);
+        e = __fmaf_rn(dc->far_l[0], wx, e);
+        f = __fmaf_rn(dc->far_l[1], wy, f);
+        two_sum(p, q, s, t);
+        t = __fadd_rn(t, __fadd_rn(e, f));
+        r.x = __fadd_rn(s, t);
+        r.y = __fsub_rn(t, __fsub_rn(r.x, s));
+    } else {
+        pair_from(far_field(dc, ix, iy, half), r.x, r.y);
     }
-    r2 = block_sum0<M>(r2, sh);
-    b2 = block_sum0<M>(b2, sh);
-    if (threadIdx.x == 0) {
-        Slot* red = static_cast<Slot*>(dc->mg_red);
-        red[2 * (size_t)tr.slot] = r2.slot();
-        red[2 * (size_t)tr.slot + 1] = b2.slot();
+    return r;
+}
+
+// A case's cells as the residual sees them: wall ghosts hold the wall value and the inner
+// cell's coefficient.
+template <class M>
+__device__ __forceinline__ PotCell<M> pot_cell(const DevCase* dc, unsigned k) {
+    PotCell<M> c;
+    if constexpr (sizeof(M) == 8) {
+        c.v = dc->phi64[k];
+    } else {
+        c.v = static_cast<const float*>(dc->phi)[k];
+        c.lo = dc->phi_lo[k];
+    }
+    c.mu = static_cast<const M*>(dc->lev[0].mu)[k];
+    return c;
+}
+template <class M>
+__device__ __forceinline__ void set_wall(PotCell<M>& c, const DevCase* dc, int ix, int iy, int half) {
+    if constexpr (sizeof(M) == 8) {
+        c.v = far_field(dc, ix, iy, half);
+    } else {
+        const float2 w = far_pair(dc, ix, iy, half);
+        c.v = w.x;
+        c.lo = w.y;
     }
 }
+
+// The face terms of a cell from its left and lower neighbours; fx, fy: 1/2 for a face between
+// cells, 1 for a face to a Dirichlet wall (mu is the inner cell's on both sides), 0 for one to
+// an insulating wall.
+__device__ __forceinline__ FaceTerm<double> face_terms(const PotCell<double>& c, const PotCell<double>& l,
+                                                       const PotCell<double>& b, double fx, double fy) {
+    FaceTerm<double> t;
+    t.x = fx * (c.mu + l.mu) * (c.v - l.v);
+    t.y = fy * (c.mu + b.mu) * (c.v - b.v);
+    return t;
+}
+__device__ __forceinline__ FaceTerm<float> face_terms(const PotCell<float>& c, const PotCell<float>& l,
+                                                      const PotCell<float>& b, float fx, float fy) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 k = __fmul2_rn(make_float2(fx, fy), __fadd2_rn(make_float2(c.mu, c.mu), make_float2(l.mu, b.mu)));
+    float2 d, e;
+    two_sum2(make_float2(c.v, c.v), __fmul2_rn(make_float2(l.v, b.v), m1), d, e);
+    e = __fadd2_rn(e, __ffma2_rn(make_float2(l.lo, b.lo), m1, make_float2(c.lo, c.lo)));
+    FaceTerm<float> t;
+    t.h = __fmul2_rn(k, d);
+    t.l = __ffma2_rn(k, e, __ffma2_rn(k, d, __fmul2_rn(t.h, m1)));
+    return t;
+}
+__device__ __forceinline__ double shfl_right(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ float shfl_right(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
 // The one call of cudaGraphSetConditional of a check: every case adds one to the ticket
 // after it has added its vote to not_done; the last one sets the loop condition (run
 // another cycle while a case still needs one) and clears both counters.
 __device__ __forceinline__ void decide_next_cycle(int* not_done, unsigned* ticket, int ncases,
                                                   cudaGraphConditionalHandle cond) {
+    if (ncases == 1) {   // the only case is done (decide() handles one that is not)
+        cudaGraphSetConditional(cond, 0u);
+        return;
+    }
     __threadfence();
     if (atomicAdd(ticket, 1u) == (unsigned)(ncases - 1)) {
         __threadfence();
@@ -285,102 +268,247 @@ __device__ __forceinline__ void decide_next_cycle(int* not_done, unsigned* ticke
     }
 }
 
-// relative residual, convergence flag, cycle count: kFinChunks blocks per case sum
-// fixed contiguous ranges of the tile partials; the last block to finish (a ticket,
-// no waiting) sums the chunk sums in chunk order and decides.  first: the step's
-// first check (resets the cycle count); later checks skip converged cases.  A case
-// that has not converged gets another cycle unless it has had kmax, in which case it
-// is marked as failed and left alone.  set_cond: inside a conditional graph, the last
-// case to decide sets whether the loop runs another cycle.
-template <class M>
-__global__ void k_mg_finalize(const DevCase* __restrict__ cases, const int* __restrict__ ids, double tol,
-                              int first, int kmax, int* not_done, unsigned* ticket, int ncases,
-                              cudaGraphConditionalHandle cond, int set_cond) {
-    using Slot = typename DSum<M>::Slot;
-    __shared__ Slot sh[32];
-    __shared__ bool last;
-    const DevCase* dc = cases + ids[blockIdx.y];
-    if (!first && pot_done(dc)) {
-        if (set_cond && blockIdx.x == 0 && threadIdx.x == 0) decide_next_cycle(not_done, ticket, ncases, cond);
-        return;
-    }
-    const int T = dc->mg_tiles, c = blockIdx.x;
-    const int t0 = (int)((long long)T * c / kFinChunks), t1 = (int)((long long)T * (c + 1) / kFinChunks);
-    const Slot* red = static_cast<const Slot*>(dc->mg_red);
-    DSum<M> r2 = DSum<M>::zero(), b2 = DSum<M>::zero();
-    for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
-        r2.add(DSum<M>::of(red[2 * (size_t)t]));
-        b2.add(DSum<M>::of(red[2 * (size_t)t + 1]));
-    }
-    r2 = block_sum0<M>(r2, sh);
-    b2 = block_sum0<M>(b2, sh);
-    Slot* ch = static_cast<Slot*>(dc->chunk) + kFinChunks * kRedN;
-    if (threadIdx.x == 0) {
-        ch[2 * c] = r2.slot();
-        ch[2 * c + 1] = b2.slot();
-        __threadfence();
-        last = atomicAdd(&dc->tickets[1], 1u) == (unsigned)(kFinChunks - 1);
-    }
-    __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
-    __threadfence();
-    // the chunk sums, one per lane, combined by a fixed shuffle tree (the same order
-    // whichever block is last)
-    static_assert(kFinChunks <= 32, "one chunk per lane");
-    const int lane = threadIdx.x;
-    DSum<M> R2 = lane < kFinChunks ? DSum<M>::of(ld_cg(&ch[2 * lane])) : DSum<M>::zero();
-    DSum<M> B2 = lane < kFinChunks ? DSum<M>::of(ld_cg(&ch[2 * lane + 1])) : DSum<M>::zero();
-    for (int o = 16; o > 0; o >>= 1) {
-        R2.shfl_add(o);
-        B2.shfl_add(o);
-    }
-    if (lane != 0) return;
-    dc->tickets[1] = 0u;
-    const double rr = R2.value(), bb = B2.value();
-    const double rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
+// The relative residual of a case is known: converged, failed, or one cycle more.  A case that
+// has not converged gets another cycle unless it has had kmax, in which case it is marked as
+// failed and left alone.  first: the step's first check (resets the cycle count).
+__device__ __forceinline__ void decide(const DevCase* dc, const PotCheck& ck, double rr, double bb, bool scaled) {
     double* st = dc->stats;
+    const double rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
     st[ST_POT_RESID] = rel;
-    const bool done = rel <= tol;
-    if (first) st[ST_POT_CYCLES] = 0.0;
-    if (done) {
+    if (ck.first) {
+        st[ST_POT_CYCLES] = 0.0;
+        st[ST_EXTRAP] = 1.0;   // from now on phi_prev holds a step's potential (FP64)
+    }
+    if (rel <= ck.tol) {
         st[ST_POT_DONE] = 1.0;
-    } else if (st[ST_POT_CYCLES] >= (double)kmax) {
+    } else if (st[ST_POT_CYCLES] >= (double)ck.kmax) {
         st[ST_POT_FAIL] = 1.0;
         st[ST_POT_DONE] = 1.0;   // no further kernel of this step touches the case
     } else {
         st[ST_POT_DONE] = 0.0;
         st[ST_POT_CYCLES] += 1.0;
-        atomicAdd(not_done, 1);
+        if (scaled) {   // the power of two that brings the root-mean-square residual to about 1
+            int ex = 0;
+            const double rms = sqrt(rr / ((double)dc->P.nx * dc->P.ny));
+            if (rms > 0.0 && isfinite(rms)) frexp(rms, &ex);
+            st[ST_SCALE] = ldexp(1.0, ex < -1000 ? 1000 : -ex);
+        }
+        if (ck.set_cond && ck.ncases == 1) {
+            cudaGraphSetConditional(ck.cond, 1u);
+            return;
+        }
+        atomicAdd(ck.not_done, 1);
     }
-    if (set_cond) decide_next_cycle(not_done, ticket, ncases, cond);
+    if (ck.set_cond) decide_next_cycle(ck.not_done, ck.ticket, ck.ncases, ck.cond);
+}
+
+// One warp per strip of kResidW columns and `rows` rows, one lane per column and one halo
+// column on each side, marching up in y with the next row's loads in flight; a strip's norms go
+// to its slot, and the warp that finishes last (an atomic ticket per group of strips and one per
+// case, no waiting) sums them in a fixed order and decides.  Bound by HBM on large grids
+// (16 B a cell in mixed precision, 24 in FP64), by latency on small ones.
+constexpr int kResidW = kResidStripW;
+
+template <class M>
+__global__ void __launch_bounds__(32) k_residual(const DevCase* __restrict__ cases, const TileRef* __restrict__ tiles,
+                                                 int rows, const PotCheck ck) {
+    using Slot = typename DSum<M>::Slot;
+    const TileRef tr = tiles[blockIdx.x];
+    const DevCase* dc = cases + tr.case_id;
+    const int lane = threadIdx.x;
+    if (!ck.first && pot_done(dc)) {
+        if (ck.set_cond && tr.slot == 0 && lane == 0) decide_next_cycle(ck.not_done, ck.ticket, ck.ncases, ck.cond);
+        return;
+    }
+    const CaseParams& P = dc->P;
+    const int nx = P.nx, ny = P.ny;
+    const unsigned pitch = (unsigned)P.pitch;
+    const bool per_x = P.periodic_x != 0, per_y = P.periodic_y != 0;
+    const int gx = tr.x0 - 1 + lane, y0 = tr.y0, y1 = min(y0 + rows, ny);
+    int sx = gx;
+    if (per_x) sx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+    sx = min(max(sx, 0), nx - 1);
+    const bool wall_lo = !per_x && gx == -1, wall_hi = !per_x && gx == nx;
+    // factor of the left face: between cells, to the left wall (cell 0) or to the right wall (ghost nx)
+    M fx = M(0.5);
+    if (!per_x && gx == 0) fx = P.mag_dir[0] ? M(1) : M(0);
+    if (wall_hi) fx = P.mag_dir[1] ? M(1) : M(0);
+    const bool active = lane >= 1 && lane <= kResidW && gx < nx;
+    auto load_row = [&](int j) {
+        int sy = j;
+        if (per_y) sy = j < 0 ? j + ny : (j >= ny ? j - ny : j);
+        sy = min(max(sy, 0), ny - 1);
+        return pot_cell<M>(dc, (unsigned)sy * pitch + (unsigned)sx);
+    };
+    auto ghosts = [&](PotCell<M>& c, int j) {
+        if (wall_lo || wall_hi) set_wall<M>(c, dc, wall_lo ? 0 : nx, j, 1);
+        if (!per_y && (j == -1 || j == ny)) set_wall<M>(c, dc, sx, j == -1 ? 0 : ny, 0);
+    };
+    M* r_out = static_cast<M*>(dc->lev[0].r);
+    DSum<M> r2 = DSum<M>::zero(), b2 = DSum<M>::zero();
+    const auto march = [&](auto edge_tag) {
+    constexpr bool EDGE = decltype(edge_tag)::value;   // a wall or a periodic wrap lies in the strip
+    PotCell<M> below = load_row(y0 - 1), c0 = load_row(y0), c1 = load_row(y0 + 1);   // two rows in flight
+    if (EDGE) ghosts(below, y0 - 1);
+    FaceTerm<M> prev{};      // of row j-1
+    M rx_h = 0, rx_l = 0;    // T of the right face of row j-1 (FP64: rx_h)
+    for (int j = y0; j <= y1; ++j) {
+        PotCell<M> c = c0;
+        c0 = c1;
+        if (j + 2 <= y1) c1 = load_row(j + 2);
+        if (EDGE) ghosts(c, j);
+        PotCell<M> l;
+        l.v = __shfl_up_sync(0xffffffffu, c.v, 1);
+        l.mu = __shfl_up_sync(0xffffffffu, c.mu, 1);
+        if constexpr (sizeof(M) == 4) l.lo = __shfl_up_sync(0xffffffffu, c.lo, 1);
+        M fy = M(0.5);
+        if (EDGE && !per_y && j == 0) fy = P.mag_dir[2] ? M(1) : M(0);
+        if (EDGE && !per_y && j == ny) fy = P.mag_dir[3] ? M(1) : M(0);
+        const FaceTerm<M> t = face_terms(c, l, below, EDGE ? fx : M(0.5), fy);
+        if (active && j > y0) {   // row j-1: r = (T(right) - T(left)) + (T(top) - T(bottom))
+            M r;
+            if constexpr (sizeof(M) == 8) {
+                r = (rx_h - prev.x) + (t.y - prev.y);
+            } else {
+                const float2 m1 = make_float2(-1.f, -1.f);
+                float2 s, e;
+                two_sum2(make_float2(rx_h, t.h.y), __fmul2_rn(prev.h, m1), s, e);
+                e = __fadd2_rn(e, __ffma2_rn(prev.l, m1, make_float2(rx_l, t.l.y)));
+                float h, q;
+                two_sum(s.x, s.y, h, q);
+                r = __fadd_rn(h, __fadd_rn(q, __fadd_rn(e.x, e.y)));
+            }
+            r_out[(unsigned)(j - 1) * pitch + (unsigned)gx] = r;
+            r2.add(r * r);
+            // |b|^2 of the step, at cells next to a Dirichlet wall
+            const int jj = j - 1;
+            if (EDGE && ck.first && (gx == 0 || gx == nx - 1 || jj == 0 || jj == ny - 1)) {
+                const bool on[4] = {!per_x && gx == 0 && P.mag_dir[0], !per_x && gx == nx - 1 && P.mag_dir[1],
+                                    !per_y && jj == 0 && P.mag_dir[2], !per_y && jj == ny - 1 && P.mag_dir[3]};
+                DSum<M> b = DSum<M>::zero();
+#pragma unroll
+                for (int w = 0; w < 4; ++w)
+                    if (on[w]) {
+                        const int ix = w == 1 ? nx : (w == 0 ? 0 : gx), iy = w == 3 ? ny : (w == 2 ? 0 : jj);
+                        if constexpr (sizeof(M) == 8) b.add(far_field(dc, ix, iy, w < 2));
+                        else b.add(far_pair(dc, ix, iy, w < 2));
+                    }
+                const M m2 = M(2) * below.mu;   // `below` is row j-1, this cell
+                if constexpr (sizeof(M) == 8) {
+                    const double v = m2 * b.v;
+                    b2.add(v * v);
+                } else {
+                    float h, l, q, ql;
+                    two_prod(m2, b.v.x, h, l);
+                    l = __fmaf_rn(m2, b.v.y, l);
+                    two_prod(h, h, q, ql);
+                    b2.add(make_float2(q, __fmaf_rn(2.f * h, l, ql)));
+                }
+            }
+        }
+        prev = t;
+        if constexpr (sizeof(M) == 8) {
+            rx_h = shfl_right(t.x);
+        } else {
+            rx_h = shfl_right(t.h.x);
+            rx_l = shfl_right(t.l.x);
+        }
+        below = c;
+    }
+    };
+    if (tr.x0 >= 1 && tr.x0 + kResidW < nx && y0 >= 1 && y1 < ny) march(std::false_type{});
+    else march(std::true_type{});
+    for (int o = 16; o > 0; o >>= 1) {
+        r2.shfl_add(o);
+        b2.shfl_add(o);
+    }
+    Slot* red = static_cast<Slot*>(dc->mg_red);
+    Slot* groups = static_cast<Slot*>(dc->mg_groups);
+    if (lane == 0) {
+        red[2 * (size_t)tr.slot] = r2.slot();
+        red[2 * (size_t)tr.slot + 1] = b2.slot();
+    }
+    const int strips = dc->mg_strips;
+    const int size = strips <= 1024 ? 1024 : kStageGroup;
+    const int g = tr.slot / size, ng = (strips + size - 1) / size, n = min(size, strips - g * size);
+    auto sum2 = [&](const Slot* s, int m, DSum<M>& a, DSum<M>& b) {
+        a = b = DSum<M>::zero();
+        for (int t = lane; t < m; t += 32) {
+            a.add(DSum<M>::of(ld_cg(&s[2 * (size_t)t])));
+            b.add(DSum<M>::of(ld_cg(&s[2 * (size_t)t + 1])));
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            a.shfl_add(o);
+            b.shfl_add(o);
+        }
+    };
+    if (!last_of(&dc->mg_tickets[1 + g], n, lane)) return;
+    sum2(red + 2 * (size_t)g * size, n, r2, b2);
+    if (ng > 1) {
+        if (lane == 0) {
+            groups[2 * (size_t)g] = r2.slot();
+            groups[2 * (size_t)g + 1] = b2.slot();
+        }
+        if (!last_of(&dc->mg_tickets[0], ng, lane)) return;
+        sum2(groups, ng, r2, b2);
+    }
+    if (lane != 0) return;
+    if (ck.first) dc->stats[ST_B2] = b2.value();
+    decide(dc, ck, r2.value(), ck.first ? b2.value() : dc->stats[ST_B2], sizeof(M) == 8);
+}
+
+// A case's walls as one word held in a register: bits 0-3 Dirichlet walls, 4 and 5 periodic axes.
+__device__ __forceinline__ int wall_mask(const CaseParams& P) {
+    return (P.mag_dir[0] ? 1 : 0) | (P.mag_dir[1] ? 2 : 0) | (P.mag_dir[2] ? 4 : 0) | (P.mag_dir[3] ? 8 : 0) |
+           (P.periodic_x ? 16 : 0) | (P.periodic_y ? 32 : 0);
 }
 
 // coarse value at (I, J), possibly one cell outside: periodic wrap, Dirichlet wall
 // (homogeneous) mirrors with a sign change, an insulating wall mirrors evenly
 template <class M>
-__device__ __forceinline__ M coarse_at(const CaseParams& P, const M* e, int nx, int ny, int pitch,
-                                       int I, int J) {
+__device__ __forceinline__ M coarse_at(int walls, const M* e, int nx, int ny, int pitch, int I, int J) {
     M sgn = M(1);
     if (I < 0 || I >= nx) {
-        if (P.periodic_x) {
+        if (walls & 16) {
             I = I < 0 ? I + nx : I - nx;
         } else {
             const int w = I < 0 ? 0 : 1;
             I = I < 0 ? 0 : nx - 1;
-            if (P.mag_dir[w]) sgn = -sgn;
+            if (walls >> w & 1) sgn = -sgn;
         }
     }
     if (J < 0 || J >= ny) {
-        if (P.periodic_y) {
+        if (walls & 32) {
             J = J < 0 ? J + ny : J - ny;
         } else {
             const int w = J < 0 ? 2 : 3;
             J = J < 0 ? 0 : ny - 1;
-            if (P.mag_dir[w]) sgn = -sgn;
+            if (walls >> w & 1) sgn = -sgn;
         }
     }
     return sgn * e[(unsigned)J * (unsigned)pitch + (unsigned)I];
 }
+
+// scale of the fine level's residual on its way into the FP32 correction (FP64 mode)
+template <class S>
+__device__ __forceinline__ S pot_scale(const DevCase* dc) {
+    if constexpr (sizeof(S) == 8) return dc->stats[ST_SCALE];
+    else return 1.0f;
+}
+// phi += e: in FP64, or as a renormalised FP32 pair
+template <class M0>
+__device__ __forceinline__ void add_correction(const DevCase* dc, unsigned k, float e) {
+    if constexpr (sizeof(M0) == 8) {
+        dc->phi64[k] += (double)e / dc->stats[ST_SCALE];   // (a power of two)
+    } else {
+        float* hi = static_cast<float*>(dc->phi);
+        float h = hi[k], l = dc->phi_lo[k];
+        pair_add(h, l, e, 0.f);
+        hi[k] = h;
+        dc->phi_lo[k] = l;
+    }
+}
+
 
 // ---- fused V-cycle legs ------------------------------------------------------
 // A block owns a TX x TY tile of one level (32 x 16, or 16 x 8 on levels with too few
@@ -424,7 +552,7 @@ __device__ __forceinline__ int region_source(const CaseParams& P, int nx, int ny
 // neighbour sum: A x = diag x_k - off.  Regular levels take the plain five-point
 // coefficients; a ragged level the geometric factors of its narrower last cells.
 template <class M, int TX, int TY, int H>
-__device__ __forceinline__ void region_stencil(const CaseParams& P, const MGLevel& lv, int x0, int y0,
+__device__ __forceinline__ void region_stencil(int dirichlet, const MGLevel& lv, int x0, int y0,
                                                const M* mu, const M* x, const unsigned char* in, int k,
                                                M& diag, M& off) {
     using G = FRegion<TX, TY, H>;
@@ -439,7 +567,7 @@ __device__ __forceinline__ void region_stencil(const CaseParams& P, const MGLeve
                 const M mf = M(0.5) * (mc + mu[kn]);
                 diag += mf;
                 off += mf * x[kn];
-            } else if (P.mag_dir[w]) {
+            } else if (dirichlet >> w & 1) {
                 diag += M(2) * mc;
             }
         }
@@ -453,7 +581,7 @@ __device__ __forceinline__ void region_stencil(const CaseParams& P, const MGLeve
             const M mf = face_factor<M>(lv, gx, gy, w, false) * M(0.5) * (mc + mu[kn]);
             diag += mf;
             off += mf * x[kn];
-        } else if (P.mag_dir[w]) {
+        } else if (dirichlet >> w & 1) {
             diag += face_factor<M>(lv, gx, gy, w, true) * mc;
         }
     }
@@ -461,7 +589,7 @@ __device__ __forceinline__ void region_stencil(const CaseParams& P, const MGLeve
 
 // (A x) at region cell k in difference form, sum_f g mu_f (x_k - x_nb) + walls
 template <class M, int TX, int TY, int H>
-__device__ __forceinline__ M region_apply(const CaseParams& P, const MGLevel& lv, int x0, int y0, const M* mu,
+__device__ __forceinline__ M region_apply(int dirichlet, const MGLevel& lv, int x0, int y0, const M* mu,
                                           const M* x, const unsigned char* in, int k) {
     using G = FRegion<TX, TY, H>;
     const M mc = mu[k], xc = x[k];
@@ -473,7 +601,7 @@ __device__ __forceinline__ M region_apply(const CaseParams& P, const MGLevel& lv
         if (in[kn]) {
             if (lv.ragged) ax += face_factor<M>(lv, gx, gy, w, false) * M(0.5) * (mc + mu[kn]) * (xc - x[kn]);
             else ax += M(0.5) * (mc + mu[kn]) * (xc - x[kn]);
-        } else if (P.mag_dir[w]) {
+        } else if (dirichlet >> w & 1) {
             ax += (lv.ragged ? face_factor<M>(lv, gx, gy, w, true) : M(2)) * mc * xc;
         }
     }
@@ -481,7 +609,7 @@ __device__ __forceinline__ M region_apply(const CaseParams& P, const MGLevel& lv
 }
 
 template <class M, int TX, int TY, int H>
-__device__ __forceinline__ void region_half_sweep(const CaseParams& P, const MGLevel& lv, int x0, int y0,
+__device__ __forceinline__ void region_half_sweep(int dirichlet, const MGLevel& lv, int x0, int y0,
                                                   const M* mu, const M* r, M* e, const unsigned char* in, int c,
                                                   int h) {
     using G = FRegion<TX, TY, H>;
@@ -494,44 +622,48 @@ __device__ __forceinline__ void region_half_sweep(const CaseParams& P, const MGL
         const int k = ly * G::W + lx;
         if (!in[k]) continue;
         M diag, off;
-        region_stencil<M, TX, TY, H>(P, lv, x0, y0, mu, e, in, k, diag, off);
+        region_stencil<M, TX, TY, H>(dirichlet, lv, x0, y0, mu, e, in, k, diag, off);
         e[k] = fdiv(r[k] + off, diag);
     }
 }
 
-template <class M, int TX, int TY, int H>
+template <class S, class M, int TX, int TY, int H>
 __device__ __forceinline__ void region_load(const CaseParams& P, const MGLevel& lv, int x0, int y0, M* smu,
-                                            M* sr, M* se, unsigned char* in, bool load_e) {
+                                            M* sr, M* se, unsigned char* in, bool load_e, S scale) {
     using G = FRegion<TX, TY, H>;
-    const M* mu = static_cast<const M*>(lv.mu);
-    const M* r = static_cast<const M*>(lv.r);
+    const S* mu = static_cast<const S*>(lv.mu);
+    const S* r = static_cast<const S*>(lv.r);
     const M* e = static_cast<const M*>(lv.e);
     for (int k = threadIdx.x; k < G::N; k += blockDim.x) {
         int gx, gy, sx, sy;
         const int ok = region_source(P, lv.nx, lv.ny, x0, y0, H, G::W, k, gx, gy, sx, sy);
         const unsigned g = (unsigned)sy * (unsigned)lv.pitch + (unsigned)sx;
         in[k] = (unsigned char)ok;
-        smu[k] = ok ? mu[g] : M(0);
-        sr[k] = ok ? r[g] : M(0);
+        smu[k] = ok ? M(mu[g]) : M(0);
+        sr[k] = ok ? (sizeof(S) == 8 ? M(r[g] * scale) : M(r[g])) : M(0);
         se[k] = (ok && load_e) ? e[g] : M(0);
     }
 }
 
-template <class M, int TX, int TY>
+// S: the type in which the level keeps mu and r (double on the fine level of the FP64 mode,
+// whose residual enters scaled); everything else is FP32.
+template <class S, int TX, int TY>
 __global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases,
                                                const TileRef* __restrict__ tiles, int L) {
+    using M = float;
     using G = FRegion<TX, TY, kHD>;
     __shared__ M smu[G::N], sr[G::N], se[G::N];
     __shared__ unsigned char in[G::N];
     const TileRef tr = tiles[blockIdx.x];
     const DevCase* dc = cases + tr.case_id;
-    if (pot_done(dc) || L >= dc->nlev - 1) return;
+    if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
+    const int dirichlet = wall_mask(P);
     const MGLevel lv = dc->lev[L], cv = dc->lev[L + 1];
-    region_load<M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, sr, se, in, false);
+    region_load<S, M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, sr, se, in, false, pot_scale<S>(dc));
     __syncthreads();
     for (int h = 1; h <= 2 * kFNu; ++h) {
-        region_half_sweep<M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
+        region_half_sweep<M, TX, TY, kHD>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
         __syncthreads();
     }
     // pre-smoothed correction of the tile
@@ -569,15 +701,18 @@ __global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases
             const int lx = kHD + 2 * ci + (q & 1), ly = kHD + 2 * cj + (q >> 1);
             const int k = ly * G::W + lx;
             if (!in[k]) continue;
-            acc += sr[k] - region_apply<M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, se, in, k);
+            acc += sr[k] - region_apply<M, TX, TY, kHD>(dirichlet, lv, tr.x0, tr.y0, smu, se, in, k);
         }
         rc[(unsigned)J * (unsigned)cv.pitch + (unsigned)I] = acc;
     }
 }
 
-template <class M, int TX, int TY>
+// FINE: the fine level, where the smoothed correction goes straight into the master potential
+// (M0: its precision) instead of back to e.
+template <class S, class M0, bool FINE, int TX, int TY>
 __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
                                              const TileRef* __restrict__ tiles, int L) {
+    using M = float;
     using G = FRegion<TX, TY, kHU>;
     constexpr int CW = (TX + 2 * kHU) / 2 + 3, CH = (TY + 2 * kHU) / 2 + 3;
     __shared__ M smu[G::N], sr[G::N], se[G::N];
@@ -585,10 +720,11 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
     __shared__ unsigned char in[G::N];
     const TileRef tr = tiles[blockIdx.x];
     const DevCase* dc = cases + tr.case_id;
-    if (pot_done(dc) || L >= dc->nlev - 1) return;
+    if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
+    const int dirichlet = wall_mask(P);
     const MGLevel lv = dc->lev[L], cv = dc->lev[L + 1];
-    region_load<M, TX, TY, kHU>(P, lv, tr.x0, tr.y0, smu, sr, se, in, true);
+    region_load<S, M, TX, TY, kHU>(P, lv, tr.x0, tr.y0, smu, sr, se, in, true, pot_scale<S>(dc));
     // coarse corrections around the region (one cell beyond its parents)
     const int cx0 = (tr.x0 - kHU) / 2 - 1 - ((tr.x0 - kHU) < 0 ? 1 : 0);
     const int cy0 = (tr.y0 - kHU) / 2 - 1 - ((tr.y0 - kHU) < 0 ? 1 : 0);
@@ -601,7 +737,7 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
         else I = I < -1 ? -1 : (I > cv.nx ? cv.nx : I);
         if (P.periodic_y) J = ((J % cv.ny) + cv.ny) % cv.ny;
         else J = J < -1 ? -1 : (J > cv.ny ? cv.ny : J);
-        sc[k] = coarse_at<M>(P, ec, cv.nx, cv.ny, cv.pitch, I, J);
+        sc[k] = coarse_at<M>(dirichlet, ec, cv.nx, cv.ny, cv.pitch, I, J);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < G::N; k += blockDim.x) {
@@ -627,21 +763,27 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
     }
     __syncthreads();
     for (int h = 1; h <= 2 * kFNu; ++h) {
-        region_half_sweep<M, TX, TY, kHU>(P, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
+        region_half_sweep<M, TX, TY, kHU>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
         __syncthreads();
     }
     M* e = static_cast<M*>(lv.e);
     for (int t = threadIdx.x; t < TX * TY; t += blockDim.x) {
         const int gx = tr.x0 + t % TX, gy = tr.y0 + t / TX;
-        if (gx < lv.nx && gy < lv.ny)
-            e[(unsigned)gy * (unsigned)lv.pitch + (unsigned)gx] = se[(t / TX + kHU) * G::W + t % TX + kHU];
+        if (gx < lv.nx && gy < lv.ny) {
+            const unsigned k = (unsigned)gy * (unsigned)lv.pitch + (unsigned)gx;
+            const M v = se[(t / TX + kHU) * G::W + t % TX + kHU];
+            if (FINE) add_correction<M0>(dc, k, v);
+            else e[k] = v;
+        }
     }
 }
 
 // conjugate gradients on the coarsest level, one block per case, in shared memory
-template <class M>
+// (for coarsest levels too large for the tail kernel: a periodic axis that halves to an odd
+// size early)
 __global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ cases,
                                                   const int* __restrict__ ids) {
+    using M = float;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ M red[32];
     const DevCase* dc = cases + ids[blockIdx.x];
@@ -666,10 +808,10 @@ __global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ ca
     for (int k = threadIdx.x; k < n; k += blockDim.x) rr += r[k] * r[k];
     rr = block_sum(rr, red);
     const M rr0 = rr;
-    // the coarse correction of a V-cycle needs only a few digits: FP32 stops at 1e-3
-    // relative, FP64 at 1e-6 (either way the cycle contracts as with an exact coarse
-    // solve; the fine-level residual test alone decides when the potential is converged)
-    const M tol2 = sizeof(M) == 8 ? M(1e-12) : M(1e-6);
+    // the coarse correction of a V-cycle needs only a few digits: 1e-3 relative (the cycle
+    // contracts as with an exact coarse solve; the fine-level residual test alone decides
+    // when the potential is converged)
+    const M tol2 = M(1e-6);
     const int maxit = 4 * (nx + ny) + 100;
     for (int it = 0; it < maxit && rr > tol2 * rr0 && rr > M(0); ++it) {
         M pAp = 0;
@@ -698,11 +840,23 @@ __global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ ca
     }
 }
 
-// The same solve by one warp per case, for coarsest levels of up to kCoarsestWarp
-// cells: the operator's coefficients are formed once, and an iteration's two sums are
-// warp shuffles, with no block-wide barrier.  Each iteration is a few hundred cycles
-// instead of the block version's six barriers.
-constexpr int kCoarsestWarp = 1024;
+// ---- the coarse levels in one kernel ---------------------------------------------------
+// One block per case takes the V-cycle from level dc->tail (at most kTailCells cells) down to
+// the coarsest level and back, all in shared memory: on small levels a kernel per leg is all
+// launch latency.  Red-black Gauss-Seidel sweeps, restriction and prolongation are those of the
+// fused legs; the face coefficients and the inverse diagonal are formed once per level.  Levels
+// of at most kWarpCells cells are swept by one warp, without block barriers.  The coarsest
+// level is swept 2 kFNu times when it has at most kTinyCells cells and solved by conjugate
+// gradients otherwise (grids whose one axis runs out first).  The part of at most kPassCells cells
+// takes the block's first kTailFew threads and runs twice, so that it stands for an exact solve: with one pass the potential's error at the
+// same residual is half as large again.  A case whose tail starts at
+// level 0 adds the correction to its potential here.
+constexpr int kTailNT = 1024, kTailFew = 256, kTailPasses = 2, kTinyCells = 16;
+
+struct TailLevel {
+    int nx, ny, off, ragged;   // off: of its cells in the arrays below
+    int tab;                   // of its cells in the neighbour table (levels of one warp), or -1
+};
 
 template <class M>
 __device__ __forceinline__ M warp_allsum(M v) {
@@ -711,118 +865,327 @@ __device__ __forceinline__ M warp_allsum(M v) {
     return v;
 }
 
-template <class M>
-__global__ void __launch_bounds__(32) k_coarsest_warp(const DevCase* __restrict__ cases,
-                                                      const int* __restrict__ ids) {
+// cells of a level by the first nt threads' warps, row by row: f(i, j, k), cells of one colour
+// (0, 1) or all (-1)
+template <class F>
+__device__ __forceinline__ void tail_cells(int nt, int nx, int ny, int colour, F f) {
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < ny; j += nt >> 5)
+        if (colour < 0) {
+            for (int i = lane; i < nx; i += 32) f(i, j, j * nx + i);
+        } else {
+            for (int i = 2 * lane + ((colour + j) & 1); i < nx; i += 64) f(i, j, j * nx + i);
+        }
+}
+
+// barrier of the block, or of its first kTailFew threads
+__device__ __forceinline__ void tail_sync(int nt) {
+    if (nt == kTailNT) __syncthreads();
+    else asm volatile("bar.sync 1, %0;" ::"n"(kTailFew) : "memory");
+}
+
+template <class M0>
+__global__ void __launch_bounds__(kTailNT) k_tail(const DevCase* __restrict__ cases, const int* __restrict__ ids,
+                                                  int max_cells, int max_small) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ TailLevel lv[kMaxLevels];
+    __shared__ MGLevel geo[kMaxLevels];
     const DevCase* dc = cases + ids[blockIdx.x];
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
-    const MGLevel lv = dc->lev[dc->nlev - 1];
-    const int nx = lv.nx, ny = lv.ny, n = nx * ny;
-    const int lane = threadIdx.x;
-    // x, r, p, A p, the diagonal and the four off-diagonal coefficients per cell, then
-    // the four neighbour indices (a wall side points at the cell itself with a zero
-    // coefficient)
-    M* x = reinterpret_cast<M*>(smem_raw);
-    M* r = x + n;
-    M* p = r + n;
-    M* Ap = p + n;
-    M* dg = Ap + n;
-    M* cw = dg + n;                                        // [4][n]
-    short* nb = reinterpret_cast<short*>(cw + 4 * n);       // [4][n]
-    const M* gmu = static_cast<const M*>(lv.mu);
-    M rr = 0;
-    for (int k = lane; k < n; k += 32) {
-        const int i = k % nx, j = k / nx;
-        const M mc = gmu[(size_t)j * lv.pitch + i];
-        M d = 0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            int ii, jj;
-            M c = 0;
-            int kn = k;
-            if (neighbour(P, nx, ny, i, j, w, ii, jj)) {
-                kn = jj * nx + ii;
-                c = M(0.5) * (mc + gmu[(size_t)jj * lv.pitch + ii]);
-                if (lv.ragged) c *= face_factor<M>(lv, i, j, w, false);
-                d += c;
-            } else if (P.mag_dir[w]) {
-                d += (lv.ragged ? face_factor<M>(lv, i, j, w, true) : M(2)) * mc;
-            }
-            cw[w * n + k] = c;
-            nb[w * n + k] = (short)kn;
+    const int L0 = dc->tail, n_lev = dc->nlev - L0;
+    // per level, cell by cell: mu, right-hand side, correction, coefficients of the right and
+    // upper faces (0 at a wall), inverse diagonal; p and A p of the conjugate gradients; the
+    // neighbour table: cells to the left, right, below, above, and i, j
+    float* mu = reinterpret_cast<float*>(smem_raw);
+    float *r = mu + max_cells, *e = r + max_cells, *cx = e + max_cells, *cy = cx + max_cells, *di = cy + max_cells;
+    float *p = di + max_cells, *Ap = p + max_small;
+    unsigned short* tab = reinterpret_cast<unsigned short*>(Ap + max_small);   // [max_small][6]
+    if (threadIdx.x < n_lev) {
+        int off = 0, tb = 0;
+        for (int l = 0; l < (int)threadIdx.x; ++l) {
+            const int n = dc->lev[L0 + l].nx * dc->lev[L0 + l].ny;
+            off += n;
+            if (n <= kWarpCells) tb += n;
         }
-        dg[k] = d;
-        const M rk = static_cast<const M*>(lv.r)[(size_t)j * lv.pitch + i];
-        r[k] = rk;
-        p[k] = rk;
-        x[k] = 0;
-        rr += rk * rk;
+        const MGLevel g = dc->lev[L0 + threadIdx.x];
+        geo[threadIdx.x] = g;
+        lv[threadIdx.x] = TailLevel{g.nx, g.ny, off, g.ragged,
+                                    g.nx * g.ny <= kWarpCells || (int)threadIdx.x == n_lev - 1 ? tb : -1};
     }
-    rr = warp_allsum(rr);
-    __syncwarp();
-    const M rr0 = rr;
-    // the same stopping rule as the block version
-    const M tol2 = sizeof(M) == 8 ? M(1e-12) : M(1e-6);
-    const int maxit = 4 * (nx + ny) + 100;
-    for (int it = 0; it < maxit && rr > tol2 * rr0 && rr > M(0); ++it) {
-        M pAp = 0;
-        for (int k = lane; k < n; k += 32) {
-            M a = dg[k] * p[k];
-#pragma unroll
-            for (int w = 0; w < 4; ++w) a -= cw[w * n + k] * p[nb[w * n + k]];
-            Ap[k] = a;
-            pAp += p[k] * a;
-        }
-        pAp = warp_allsum(pAp);
-        const M alpha = rr / pAp;
-        M rn = 0;
-        for (int k = lane; k < n; k += 32) {
-            x[k] += alpha * p[k];
-            const M rk = r[k] - alpha * Ap[k];
-            r[k] = rk;
-            rn += rk * rk;
-        }
-        rn = warp_allsum(rn);
-        const M beta = rn / rr;
-        rr = rn;
-        __syncwarp();   // every lane's reads of p for A p are done
-        for (int k = lane; k < n; k += 32) p[k] = r[k] + beta * p[k];
-        __syncwarp();
-    }
-    for (int k = lane; k < n; k += 32) {
-        const int i = k % nx, j = k / nx;
-        static_cast<M*>(lv.e)[(size_t)j * lv.pitch + i] = x[k];
-    }
-}
-
-template <class M>
-__global__ void __launch_bounds__(kNT) k_correct(const DevCase* __restrict__ cases,
-                                                 const TileRef* __restrict__ tiles) {
-    const TileRef tr = tiles[blockIdx.x];
-    const DevCase* dc = cases + tr.case_id;
-    if (pot_done(dc)) return;
-    const MGLevel lv = dc->lev[0];
-    const int i = tr.x0 + threadIdx.x % kMgTX;
-    if (i >= lv.nx) return;
-#pragma unroll
-    for (int q = 0; q < kRowsPT; ++q) {
-        const int j = tr.y0 + threadIdx.x / kMgTX + q * (kNT / kMgTX);
-        if (j >= lv.ny) break;
-        const unsigned k = (unsigned)j * (unsigned)lv.pitch + (unsigned)i;
-        if (sizeof(M) == 8) {
-            const double v = dc->phi64[k] + (double)static_cast<const M*>(lv.e)[k];
-            dc->phi64[k] = v;
+    {
+        const MGLevel& g = dc->lev[L0];
+        if (sizeof(M0) == 8 && L0 == 0) {
+            const double sc = dc->stats[ST_SCALE];
+            tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
+                const size_t q = (size_t)j * g.pitch + i;
+                mu[k] = (float)static_cast<const double*>(g.mu)[q];
+                r[k] = (float)(static_cast<const double*>(g.r)[q] * sc);
+            });
         } else {
-            // (phi, phi_lo) += e as a renormalised FP32 pair
-            float* hi = static_cast<float*>(dc->phi);
-            float h = hi[k], l = dc->phi_lo[k];
-            pair_add(h, l, (float)static_cast<const M*>(lv.e)[k], 0.f);
-            hi[k] = h;
-            dc->phi_lo[k] = l;
+            tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
+                const size_t q = (size_t)j * g.pitch + i;
+                mu[k] = static_cast<const float*>(g.mu)[q];
+                r[k] = static_cast<const float*>(g.r)[q];
+            });
         }
     }
+    const int walls = wall_mask(P), dirichlet = walls & 15;
+    const bool per_x = (walls & 16) != 0, per_y = (walls & 32) != 0;
+    __syncthreads();
+    // mu of the coarser levels: the mean of the children
+    for (int l = 0; l + 1 < n_lev; ++l) {
+        const TailLevel v = lv[l], c = lv[l + 1];
+        const float* m = mu + v.off;
+        tail_cells(kTailNT, c.nx, c.ny, -1, [&](int I, int J, int K) {
+            const int i0 = 2 * I, j0 = 2 * J, i1 = i0 + 1 < v.nx, j1 = j0 + 1 < v.ny;
+            const float* q = m + j0 * v.nx + i0;
+            float s = q[0];
+            if (i1) s += q[1];
+            if (j1) s += i1 ? q[v.nx] + q[v.nx + 1] : q[v.nx];
+            mu[c.off + K] = s * (i1 && j1 ? 0.25f : (i1 || j1 ? 0.5f : 1.f));
+        });
+        __syncthreads();
+    }
+    // coefficients of every level, and its neighbour table
+    for (int l = 0; l < n_lev; ++l) {
+        const TailLevel v = lv[l];
+        const MGLevel& g = geo[l];
+        const float* m = mu + v.off;
+        tail_cells(kTailNT, v.nx, v.ny, -1, [&](int i, int j, int k) {
+            const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
+            const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
+            const int kn[4] = {kl, kr, kb, kt};
+            const bool in[4] = {per_x || i > 0, per_x || i < v.nx - 1, per_y || j > 0, per_y || j < v.ny - 1};
+            const float mc = m[k];
+            float d = 0.f, c4[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                c4[w] = 0.f;
+                if (in[w]) {
+                    c4[w] = 0.5f * (mc + m[kn[w]]);
+                    if (v.ragged) c4[w] *= face_factor<float>(g, i, j, w, false);
+                    d += c4[w];
+                } else if (dirichlet >> w & 1) {
+                    d += (v.ragged ? face_factor<float>(g, i, j, w, true) : 2.f) * mc;
+                }
+            }
+            cx[v.off + k] = c4[1];
+            cy[v.off + k] = c4[3];
+            di[v.off + k] = fdiv(1.f, d);
+            if (v.tab >= 0) {
+                unsigned short* t = tab + 6 * (v.tab + k);
+                t[0] = (unsigned short)kl;
+                t[1] = (unsigned short)kr;
+                t[2] = (unsigned short)kb;
+                t[3] = (unsigned short)kt;
+                t[4] = (unsigned short)i;
+                t[5] = (unsigned short)j;
+            }
+        });
+    }
+    __syncthreads();
+    // sum_f c_f x_nb over a cell's faces (a wall face's coefficient is 0: the right face of the
+    // last column, the upper face of the last row)
+    auto nb_sum = [&](const TailLevel& v, const float* x, int k, int kl, int kr, int kb, int kt) {
+        const float *a = cx + v.off, *b = cy + v.off;
+        return (a[kl] * x[kl] + a[k] * x[kr]) + (b[kb] * x[kb] + b[k] * x[kt]);
+    };
+    // r - A x in differences, so that smooth x keeps its digits
+    auto residual = [&](const TailLevel& v, const MGLevel& g, const float* x, int i, int j, int k) {
+        const float *a = cx + v.off, *b = cy + v.off;
+        const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
+        const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
+        const float xc = x[k];
+        float ax = (a[kl] * (xc - x[kl]) + a[k] * (xc - x[kr])) + (b[kb] * (xc - x[kb]) + b[k] * (xc - x[kt]));
+        const bool at[4] = {!per_x && i == 0, !per_x && i == v.nx - 1, !per_y && j == 0, !per_y && j == v.ny - 1};
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+            if (at[w] && (dirichlet >> w & 1)) ax += (v.ragged ? face_factor<float>(g, i, j, w, true) : 2.f) * mu[v.off + k] * xc;
+        return r[v.off + k] - ax;
+    };
+    auto restrict_cell = [&](int l, int I, int J) {
+        const TailLevel v = lv[l];
+        float acc = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = 2 * I + (q & 1), j = 2 * J + (q >> 1);
+            if (i < v.nx && j < v.ny) acc += residual(v, geo[l], e + v.off, i, j, j * v.nx + i);
+        }
+        return acc;
+    };
+    auto prolong_cell = [&](int l, int i, int j) {
+        const TailLevel v = lv[l], c = lv[l + 1];
+        const float* xc = e + c.off;
+        const int I = i >> 1, J = j >> 1;
+        int di_ = (i & 1) ? 1 : -1, dj_ = (j & 1) ? 1 : -1;
+        float wx = 0.25f, wy = 0.25f;
+        if (v.ragged || c.ragged) {
+            prolong_axis<float>(i, v.nx, geo[l].wlx, c.nx, geo[l + 1].wlx, di_, wx);
+            prolong_axis<float>(j, v.ny, geo[l].wly, c.ny, geo[l + 1].wly, dj_, wy);
+        }
+        return ((1.f - wx) * (1.f - wy)) * xc[J * c.nx + I] +
+               (wx * (1.f - wy)) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J) +
+               ((1.f - wx) * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I, J + dj_) +
+               (wx * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J + dj_);
+    };
+    auto sweep = [&](int nt, int l, int colour) {
+        const TailLevel v = lv[l];
+        float* x = e + v.off;
+        tail_cells(nt, v.nx, v.ny, colour, [&](int i, int j, int k) {
+            const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
+            const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
+            x[k] = (r[v.off + k] + nb_sum(v, x, k, kl, kr, kb, kt)) * di[v.off + k];
+        });
+        tail_sync(nt);
+    };
+    const int lane = threadIdx.x & 31;
+    auto warp_sweep = [&](int l, int colour) {   // one warp
+        const TailLevel v = lv[l];
+        float* x = e + v.off;
+        const int n = v.nx * v.ny;
+        for (int k = lane; k < n; k += 32) {
+            const unsigned short* t = tab + 6 * (v.tab + k);
+            if (((t[4] + t[5]) & 1) == colour) x[k] = (r[v.off + k] + nb_sum(v, x, k, t[0], t[1], t[2], t[3])) * di[v.off + k];
+        }
+        __syncwarp();
+    };
+    int small = 0, twice = 0;   // first level of one warp, first level of the part that runs twice
+    while (small < n_lev - 1 && lv[small].tab < 0) ++small;
+    while (twice < n_lev - 1 && lv[twice].nx * lv[twice].ny > kPassCells) ++twice;
+    auto down = [&](int nt, int l, bool fresh) {
+        const TailLevel v = lv[l], c = lv[l + 1];
+        float* x = e + v.off;
+        if (fresh) {   // first sweep from zero: the first colour's neighbours are zero
+            tail_cells(nt, v.nx, v.ny, -1, [&](int i, int j, int k) { x[k] = ((i + j) & 1) ? 0.f : r[v.off + k] * di[v.off + k]; });
+            tail_sync(nt);
+        } else {
+            sweep(nt, l, 0);
+        }
+        sweep(nt, l, 1);
+        for (int s = 1; s < kFNu; ++s) {
+            sweep(nt, l, 0);
+            sweep(nt, l, 1);
+        }
+        tail_cells(nt, c.nx, c.ny, -1, [&](int I, int J, int K) { r[c.off + K] = restrict_cell(l, I, J); });
+        tail_sync(nt);
+    };
+    auto up = [&](int nt, int l) {
+        const TailLevel v = lv[l];
+        float* x = e + v.off;
+        tail_cells(nt, v.nx, v.ny, -1, [&](int i, int j, int k) { x[k] += prolong_cell(l, i, j); });
+        tail_sync(nt);
+        for (int s = 0; s < kFNu; ++s) {
+            sweep(nt, l, 0);
+            sweep(nt, l, 1);
+        }
+    };
+    auto one_warp = [&](bool fresh_top) {   // levels small to the coarsest and back
+        for (int l = small; l + 1 < n_lev; ++l) {
+            const TailLevel v = lv[l], c = lv[l + 1];
+            float* x = e + v.off;
+            const int n = v.nx * v.ny, nc = c.nx * c.ny;
+            if (fresh_top || l > small) {
+                for (int k = lane; k < n; k += 32) {
+                    const unsigned short* t = tab + 6 * (v.tab + k);
+                    x[k] = ((t[4] + t[5]) & 1) ? 0.f : r[v.off + k] * di[v.off + k];
+                }
+                __syncwarp();
+            } else {
+                warp_sweep(l, 0);
+            }
+            warp_sweep(l, 1);
+            for (int s = 1; s < kFNu; ++s) {
+                warp_sweep(l, 0);
+                warp_sweep(l, 1);
+            }
+            for (int k = lane; k < nc; k += 32) {
+                const unsigned short* t = tab + 6 * (c.tab + k);
+                r[c.off + k] = restrict_cell(l, t[4], t[5]);
+            }
+            __syncwarp();
+        }
+        const TailLevel v = lv[n_lev - 1];
+        const int n = v.nx * v.ny;
+        float *x = e + v.off, *q = r + v.off;
+        if (n <= kTinyCells) {
+            for (int k = lane; k < n; k += 32) x[k] = 0.f;
+            __syncwarp();
+            for (int s = 0; s < 2 * kFNu; ++s) {
+                warp_sweep(n_lev - 1, 0);
+                warp_sweep(n_lev - 1, 1);
+            }
+        } else {   // conjugate gradients
+            const float* dg = di + v.off;
+            float rr = 0.f;
+            for (int k = lane; k < n; k += 32) {
+                p[k] = q[k];
+                x[k] = 0.f;
+                rr += q[k] * q[k];
+            }
+            rr = warp_allsum(rr);
+            __syncwarp();
+            const float rr0 = rr;
+            const float tol2 = 1e-6f;   // a coarse correction needs only a few digits (as the block version)
+            const int maxit = 4 * (v.nx + v.ny) + 100;
+            for (int it = 0; it < maxit && rr > tol2 * rr0 && rr > 0.f; ++it) {
+                float pAp = 0.f;
+                for (int k = lane; k < n; k += 32) {
+                    const unsigned short* t = tab + 6 * (v.tab + k);
+                    const float y = fdiv(p[k], dg[k]) - nb_sum(v, p, k, t[0], t[1], t[2], t[3]);
+                    Ap[k] = y;
+                    pAp += p[k] * y;
+                }
+                pAp = warp_allsum(pAp);
+                const float alpha = rr / pAp;
+                float rn = 0.f;
+                for (int k = lane; k < n; k += 32) {
+                    x[k] += alpha * p[k];
+                    const float rk = q[k] - alpha * Ap[k];
+                    q[k] = rk;
+                    rn += rk * rk;
+                }
+                rn = warp_allsum(rn);
+                const float beta = rn / rr;
+                rr = rn;
+                __syncwarp();   // every lane's reads of p for A p are done
+                for (int k = lane; k < n; k += 32) p[k] = q[k] + beta * p[k];
+                __syncwarp();
+            }
+        }
+        for (int l = n_lev - 2; l >= small; --l) {
+            const TailLevel w = lv[l];
+            float* y = e + w.off;
+            for (int k = lane; k < w.nx * w.ny; k += 32) {
+                const unsigned short* t = tab + 6 * (w.tab + k);
+                y[k] += prolong_cell(l, t[4], t[5]);
+            }
+            __syncwarp();
+            for (int s = 0; s < kFNu; ++s) {
+                warp_sweep(l, 0);
+                warp_sweep(l, 1);
+            }
+        }
+    };
+    const int top = min(twice, small);
+    for (int l = 0; l < top; ++l) down(kTailNT, l, true);
+    if (threadIdx.x < kTailFew) {   // levels of at most kPassCells cells: the first warps
+        const int passes = twice < n_lev - 1 ? kTailPasses : 1;
+        for (int pass = 0; pass < passes; ++pass) {
+            for (int l = twice; l < small; ++l) down(kTailFew, l, pass == 0 || l > twice);
+            if (threadIdx.x < 32) one_warp(pass == 0 || small > twice);
+            tail_sync(kTailFew);
+            for (int l = small - 1; l >= twice; --l) up(kTailFew, l);
+        }
+    }
+    __syncthreads();
+    for (int l = top - 1; l >= 0; --l) up(kTailNT, l);
+    const MGLevel& g = geo[0];
+    tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
+        const unsigned q = (unsigned)j * (unsigned)g.pitch + (unsigned)i;
+        if (L0 == 0) add_correction<M0>(dc, q, e[k]);
+        else static_cast<float*>(g.e)[q] = e[k];
+    });
 }
 
 // The FP64 warm start, extrapolated linearly in time: phi <- 2 phi - phi_prev and
@@ -848,11 +1211,6 @@ __global__ void __launch_bounds__(kNT) k_extrapolate(const DevCase* __restrict__
         if (valid) dc->phi64[k] = 2.0 * v - dc->phi_prev64[k];
         dc->phi_prev64[k] = v;
     }
-}
-
-// after k_extrapolate: phi_prev of every solving case now holds this step's start
-__global__ void k_extrapolate_commit(const DevCase* __restrict__ cases, const int* __restrict__ ids, int n) {
-    for (int c = threadIdx.x; c < n; c += blockDim.x) cases[ids[c]].stats[ST_EXTRAP] = 1.0;
 }
 
 // ---- the paper's own magnetic solver (Sec. 3.2, Eqs. 12-18) ----------------------
@@ -966,105 +1324,69 @@ cudaError_t launch_pseudo_time(int prec, const DevCase* d, int nx, int ny, int i
     return cudaGetLastError();
 }
 
-cudaError_t launch_mg_residual64(int prec, const DevCase* cases, const TileRef* tiles, int n, int first,
-                                 cudaStream_t st) {
+cudaError_t launch_mg_residual(int prec, const DevCase* cases, const TileRef* tiles, int n, int rows, const PotCheck& ck,
+                               cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (prec == 0) k_residual64<double><<<n, kNT, 0, st>>>(cases, tiles, first);
-    else k_residual64<float><<<n, kNT, 0, st>>>(cases, tiles, first);
+    if (prec == 0) k_residual<double><<<n, 32, 0, st>>>(cases, tiles, rows, ck);
+    else k_residual<float><<<n, 32, 0, st>>>(cases, tiles, rows, ck);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mg_finalize(int prec, const DevCase* cases, const int* ids, int ncases, double tol, int first,
-                               int kmax, int* not_done, unsigned* ticket, cudaGraphConditionalHandle cond,
-                               int set_cond, cudaStream_t st) {
-    if (ncases <= 0) return cudaSuccess;
-    const dim3 grid(kFinChunks, ncases);
-    if (prec == 0)
-        k_mg_finalize<double><<<grid, 256, 0, st>>>(cases, ids, tol, first, kmax, not_done, ticket, ncases, cond,
-                                                    set_cond);
-    else
-        k_mg_finalize<float><<<grid, 256, 0, st>>>(cases, ids, tol, first, kmax, not_done, ticket, ncases, cond,
-                                                   set_cond);
-    return cudaGetLastError();
+template <int TX, int TY>
+static void vdown(int wide, const DevCase* cases, const TileRef* tiles, int n, int L, cudaStream_t st) {
+    constexpr int NT = TX * TY >= 512 ? 256 : 128;
+    if (wide) k_vdown<double, TX, TY><<<n, NT, 0, st>>>(cases, tiles, L);
+    else k_vdown<float, TX, TY><<<n, NT, 0, st>>>(cases, tiles, L);
 }
 
 cudaError_t launch_mg_vdown(int prec, const DevCase* cases, const TileRef* tiles, int n, int L, int small,
                             cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (small) {
-        if (prec == 0) k_vdown<double, kFusedSmallTX, kFusedSmallTY><<<n, 128, 0, st>>>(cases, tiles, L);
-        else k_vdown<float, kFusedSmallTX, kFusedSmallTY><<<n, 128, 0, st>>>(cases, tiles, L);
-    } else {
-        if (prec == 0) k_vdown<double, kFusedTX, kFusedTY><<<n, 256, 0, st>>>(cases, tiles, L);
-        else k_vdown<float, kFusedTX, kFusedTY><<<n, 256, 0, st>>>(cases, tiles, L);
-    }
+    const int wide = prec == 0 && L == 0;
+    if (small) vdown<kFusedSmallTX, kFusedSmallTY>(wide, cases, tiles, n, L, st);
+    else vdown<kFusedTX, kFusedTY>(wide, cases, tiles, n, L, st);
     return cudaGetLastError();
+}
+
+template <int TX, int TY>
+static void vup(int prec, const DevCase* cases, const TileRef* tiles, int n, int L, cudaStream_t st) {
+    constexpr int NT = TX * TY >= 512 ? 256 : 128;
+    if (L > 0) k_vup<float, float, false, TX, TY><<<n, NT, 0, st>>>(cases, tiles, L);
+    else if (prec == 0) k_vup<double, double, true, TX, TY><<<n, NT, 0, st>>>(cases, tiles, L);
+    else k_vup<float, float, true, TX, TY><<<n, NT, 0, st>>>(cases, tiles, L);
 }
 
 cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, int n, int L, int small,
                           cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (small) {
-        if (prec == 0) k_vup<double, kFusedSmallTX, kFusedSmallTY><<<n, 128, 0, st>>>(cases, tiles, L);
-        else k_vup<float, kFusedSmallTX, kFusedSmallTY><<<n, 128, 0, st>>>(cases, tiles, L);
-    } else {
-        if (prec == 0) k_vup<double, kFusedTX, kFusedTY><<<n, 256, 0, st>>>(cases, tiles, L);
-        else k_vup<float, kFusedTX, kFusedTY><<<n, 256, 0, st>>>(cases, tiles, L);
-    }
+    if (small) vup<kFusedSmallTX, kFusedSmallTY>(prec, cases, tiles, n, L, st);
+    else vup<kFusedTX, kFusedTY>(prec, cases, tiles, n, L, st);
     return cudaGetLastError();
 }
 
-size_t mg_coarsest_smem(int prec, int max_cells) {
-    const size_t m = prec == 0 ? sizeof(double) : sizeof(float);
-    if (max_cells <= kCoarsestWarp) return (size_t)9 * max_cells * m + (size_t)4 * max_cells * sizeof(short);
-    return (size_t)5 * max_cells * m;
-}
-
-cudaError_t launch_mg_coarsest(int prec, const DevCase* cases, const int* ids, int ncases,
-                               int max_cells, cudaStream_t st) {
+cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* ids, int ncases, int max_cells, int max_small,
+                           cudaStream_t st) {
     if (ncases <= 0) return cudaSuccess;
-    const size_t sm = mg_coarsest_smem(prec, max_cells);
-    const bool warp = max_cells <= kCoarsestWarp;
-    cudaError_t e;
-    if (prec == 0) {
-        if (warp) {
-            e = cudaFuncSetAttribute(k_coarsest_warp<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            k_coarsest_warp<double><<<ncases, 32, sm, st>>>(cases, ids);
-        } else {
-            e = cudaFuncSetAttribute(k_coarsest<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            k_coarsest<double><<<ncases, 256, sm, st>>>(cases, ids);
-        }
-    } else {
-        if (warp) {
-            e = cudaFuncSetAttribute(k_coarsest_warp<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            k_coarsest_warp<float><<<ncases, 32, sm, st>>>(cases, ids);
-        } else {
-            e = cudaFuncSetAttribute(k_coarsest<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-            k_coarsest<float><<<ncases, 256, sm, st>>>(cases, ids);
-        }
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, const int* ids, int ncases,
-                                  cudaStream_t st) {
-    if (n <= 0 || ncases <= 0) return cudaSuccess;
-    k_extrapolate<<<n, kNT, 0, st>>>(cases, tiles);
-    cudaError_t e = cudaGetLastError();
+    const size_t sm = (size_t)6 * max_cells * sizeof(float) + (size_t)max_small * (2 * sizeof(float) + 6 * sizeof(short));
+    auto kern = prec == 0 ? k_tail<double> : k_tail<float>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_extrapolate_commit<<<1, 128, 0, st>>>(cases, ids, ncases);
+    kern<<<ncases, kTailNT, sm, st>>>(cases, ids, max_cells, max_small);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mg_correct(int prec, const DevCase* cases, const TileRef* tiles, int n,
-                              cudaStream_t st) {
+cudaError_t launch_mg_coarsest(const DevCase* cases, const int* ids, int ncases, int max_cells, cudaStream_t st) {
+    if (ncases <= 0) return cudaSuccess;
+    const size_t sm = (size_t)5 * max_cells * sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(k_coarsest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_coarsest<<<ncases, 256, sm, st>>>(cases, ids);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if (prec == 0) k_correct<double><<<n, kNT, 0, st>>>(cases, tiles);
-    else k_correct<float><<<n, kNT, 0, st>>>(cases, tiles);
+    k_extrapolate<<<n, kNT, 0, st>>>(cases, tiles);
     return cudaGetLastError();
 }
 

@@ -357,22 +357,11 @@ __device__ __forceinline__ void sum_slots(const typename DSum<R>::Slot* s, int n
     for (int t = lane; t < n; t += 32)
 #pragma unroll
         for (int q = 0; q < kRedN; ++q) a[q].add(DSum<R>::of(ld_cg(&s[(size_t)t * kRedN + q])));
+    // a butterfly: every lane ends with the same sums
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int q = 0; q < kRedN; ++q) a[q].shfl_add(o);
+        for (int q = 0; q < kRedN; ++q) a[q].shfl_xor_add(o);
 }
-// whether this warp is the last of n to arrive at the ticket, which it then clears
-__device__ __forceinline__ bool last_of(unsigned* ticket, int n, int lane) {
-    unsigned last = 0;
-    if (lane == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == (unsigned)(n - 1);
-        if (last) *ticket = 0u;
-        __threadfence();
-    }
-    return __shfl_sync(0xffffffffu, last, 0) != 0;
-}
-
 template <class R>
 __device__ __noinline__ void finish_strip(const StageCase<R>& S, int strips, int slot, int lane, DSum<R> sumC, DSum<R> sumH,
                                           DSum<R> sumF, int nDrop, int nBad) {
@@ -402,29 +391,32 @@ __device__ __noinline__ void finish_strip(const StageCase<R>& S, int strips, int
         if (!last_of(&S.tickets[0], ng, lane)) return;
         sum_slots<R>(groups, ng, lane, a);
     }
-    if (lane != 0) return;
+    // one statistics slot per lane: FP64 instructions are slow, so each runs once for all slots
     double* st = S.stats;
-    const double drop = a[3].value(), QL = drop > 0.0 ? a[4].value() / drop : 0.0;
-    st[ST_SUM_C] = a[0].value();
-    st[ST_SUM_HE] = a[1].value();
-    st[ST_SUM_FL_DROP] = a[2].value();
-    st[ST_N_DROP] = drop;
-    st[ST_Q_L] = QL;
-    if (a[5].value() > 0.0) st[ST_NONFINITE] = 1.0;
-    const double t1 = st[ST_T] + S.dt;
-    st[ST_T] = t1;
-    st[ST_STEP] += 1.0;
+    const double old = lane < kStatN ? st[lane] : 0.0;
+    DSum<R> pick = a[0];
+    if (lane == ST_SUM_HE) pick = a[1];
+    if (lane == ST_SUM_FL_DROP) pick = a[2];
+    if (lane == ST_N_DROP) pick = a[3];
+    if (lane == ST_Q_L || lane == ST_QL_PREV) pick = a[4];
+    if (lane == ST_NONFINITE) pick = a[5];
+    double v = pick.value();
+    const double drop = __shfl_sync(0xffffffffu, v, ST_N_DROP);
+    const double QL = drop > 0.0 ? __shfl_sync(0xffffffffu, v, ST_Q_L) / drop : 0.0;
+    const double t1 = __shfl_sync(0xffffffffu, old, ST_T) + S.dt, q0 = __shfl_sync(0xffffffffu, old, ST_QL_PREV);
+    const double resid = __shfl_sync(0xffffffffu, old, ST_POT_RESID), cycles = __shfl_sync(0xffffffffu, old, ST_POT_CYCLES);
+    bool put = lane <= ST_N_DROP;
+    if (lane == ST_Q_L || lane == ST_QL_PREV) v = QL, put = true;
+    if (lane == ST_NONFINITE) put = v > 0.0, v = 1.0;
+    if (lane == ST_T) v = t1, put = true;
+    if (lane == ST_STEP || lane == ST_STEPS_CALL) v = old + 1.0, put = true;
     // freezing time: first t with Q_L >= 0.99, linear between steps
-    if (st[ST_T_FREEZE] < 0.0 && QL >= 0.99) {
-        const double q0 = st[ST_QL_PREV];
-        st[ST_T_FREEZE] = (t1 - S.dt) + S.dt * (0.99 - q0) / (QL - q0);
-    }
-    st[ST_QL_PREV] = QL;
+    if (lane == ST_T_FREEZE && old < 0.0 && QL >= 0.99) v = (t1 - S.dt) + S.dt * (0.99 - q0) / (QL - q0), put = true;
     if (S.solve_potential) {
-        st[ST_POT_RESID_MAX] = fmax(st[ST_POT_RESID_MAX], st[ST_POT_RESID]);
-        st[ST_POT_CYCLES_SUM] += st[ST_POT_CYCLES];
+        if (lane == ST_POT_RESID_MAX) v = fmax(old, resid), put = true;
+        if (lane == ST_POT_CYCLES_SUM) v = old + cycles, put = true;
     }
-    st[ST_STEPS_CALL] += 1.0;
+    if (put) st[lane] = v;
 }
 
 // Derived quantities of one row.
