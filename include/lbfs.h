@@ -60,7 +60,7 @@ typedef struct lbfs_config {
     void  (*dev_free)(void* ptr, void* user);      /* framework's caching allocator       */
     void*   alloc_user;
     int32_t mg_max_cycles;   /* refinement cycles of a potential solve after a state is set,
-                                checked on the host (0: 40)                                */
+                                checked on the device (0: 40)                              */
     double  mg_tol;          /* relative residual ||b - A phi|| / ||b|| every solve must
                                 reach (0: 1e-13 FP64, 1e-6 mixed)                          */
     int32_t tile;            /* stage-kernel strip shape id (see lbfs_autotune); 0: chosen
@@ -73,9 +73,10 @@ typedef struct lbfs_config {
                                 as a CUDA graph.  A residual still above mg_tol after the
                                 last cycle makes lbfs_step return LBFS_ENOTCONVERGED     */
     int32_t mg_plain_cycles; /* 1: launch those cycles as mg_warm_cycles plain rounds of
-                                kernels, each returning at once for a converged case,
-                                instead of a conditional graph loop (kernel profilers
-                                cannot follow conditional graph nodes); same results     */
+                                kernels, each returning at once for a converged case (those
+                                after a state is set are counted on the host), instead of
+                                one cooperative kernel for the last of them (a profiler
+                                shows their phases); same results                         */
     int32_t reserved[5];
 } lbfs_config;
 

@@ -77,11 +77,7 @@ struct lbfs_ctx {
     cudaGraph_t graph = nullptr;
     int64_t graph_launches = 0;       // kernel nodes in one recorded step, the cycle body's aside
     cudaStream_t cap_stream = nullptr; // private stream used to record the graph
-    cudaStream_t body_stream = nullptr; // private stream used to record a conditional loop body
     bool capturing = false;           // launches are being recorded into a graph
-    cudaGraphExec_t pot_exec = nullptr; // the warm potential solve as a graph, for eager steps
-    cudaGraph_t pot_graph = nullptr;
-    int64_t cycle_launches = 0;       // kernels of one refinement cycle
     // kernel timing (events on the context stream)
     bool timing = false;
     double t_ms[3] = {0, 0, 0};
@@ -124,12 +120,8 @@ void dfree(lbfs_ctx* ctx, void* p) {
 void drop_graph(lbfs_ctx* ctx) {
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
     if (ctx->graph) cudaGraphDestroy(ctx->graph);
-    if (ctx->pot_exec) cudaGraphExecDestroy(ctx->pot_exec);
-    if (ctx->pot_graph) cudaGraphDestroy(ctx->pot_graph);
     ctx->gexec = nullptr;
     ctx->graph = nullptr;
-    ctx->pot_exec = nullptr;
-    ctx->pot_graph = nullptr;
 }
 
 cudaEvent_t take_event(lbfs_ctx* ctx) {
@@ -478,146 +470,93 @@ lbfs_status vcycle(lbfs_ctx* ctx) {
     return LBFS_OK;
 }
 
+PotCheck pot_check(const lbfs_ctx* ctx, int first, int kmax, int* not_done) {
+    return PotCheck{first, ctx->mg_tol, kmax, not_done, reinterpret_cast<unsigned*>(ctx->d_flag + 1)};
+}
+
 // the residual of the master potential and each case's check
-cudaError_t check_residual(lbfs_ctx* ctx, int first, int kmax, int* not_done, unsigned* ticket,
-                           cudaGraphConditionalHandle cond, int set_cond) {
-    PotCheck ck{first, ctx->mg_tol, kmax, not_done, ticket, ctx->n_pot, cond, set_cond};
-    return launch_mg_residual(ctx->prec, ctx->d_cases, ctx->d_res_tiles, ctx->n_res_tiles, ctx->res_rows, ck, ctx->stream);
+cudaError_t check_residual(lbfs_ctx* ctx, int first, int kmax, int* not_done) {
+    return launch_mg_residual(ctx->prec, ctx->d_cases, ctx->d_res_tiles, ctx->n_res_tiles, ctx->res_rows,
+                              pot_check(ctx, first, kmax, not_done), ctx->stream);
 }
 
-// The warm potential solve, recorded into the graph being captured on ctx->stream:
-// in FP64 the linearly extrapolated start, then the step's first residual and check,
-// then a conditional WHILE node whose body is one
-// refinement cycle (V-cycle, correction, residual of the corrected potential, check).
-// The checks decide on the device whether the body runs again, so a step whose warm
-// start already meets mg_tol runs no cycle at all, and a step never runs more than
-// mg_warm_cycles.
-lbfs_status capture_warm_potential(lbfs_ctx* ctx) {
-    const int p = ctx->prec, K = ctx->mg_warm_cycles;
-    cudaStream_t s = ctx->stream;
-    int* nd = ctx->d_flag + 1;
-    unsigned* ticket = reinterpret_cast<unsigned*>(ctx->d_flag + 2);
-    cudaStreamCaptureStatus cs;
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, nullptr, nullptr, nullptr));
-    if (cs != cudaStreamCaptureStatusActive || !g) return fail(ctx, LBFS_ECUDA, "potential capture is not active");
-    cudaGraphConditionalHandle h;
-    CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
-    if (p == 0) LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
-    LK(check_residual(ctx, 1, K, nd, ticket, h, 1));
-    const cudaGraphNode_t* deps = nullptr;
-    size_t ndeps = 0;
-    CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &ndeps));
-    // (the node-parameter type has no default constructor: zeroed storage)
-    alignas(cudaGraphNodeParams) unsigned char npbuf[sizeof(cudaGraphNodeParams)];
-    std::memset(npbuf, 0, sizeof(npbuf));
-    cudaGraphNodeParams& np = *reinterpret_cast<cudaGraphNodeParams*>(npbuf);
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = h;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    cudaGraphNode_t node;
-    CK(cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &np));
-    cudaGraph_t body = np.conditional.phGraph_out[0];
-    CK(cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
-    if (!ctx->body_stream) CK(cudaStreamCreateWithFlags(&ctx->body_stream, cudaStreamNonBlocking));
-    CK(cudaStreamBeginCaptureToGraph(ctx->body_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    ctx->stream = ctx->body_stream;
-    const int64_t l0 = ctx->launches;
-    lbfs_status r = vcycle(ctx);
-    if (r == LBFS_OK) {
-        const cudaError_t e = check_residual(ctx, 0, K, nd, ticket, h, 1);
-        ++ctx->launches;
-        if (e != cudaSuccess) r = fail(ctx, LBFS_ECUDA, std::string("cycle body: ") + cudaGetErrorString(e));
+// refinement cycles until every case has converged or had kmax
+cudaError_t cycles(lbfs_ctx* ctx, int kmax) {
+    CycleArgs a{};
+    a.cases = ctx->d_cases;
+    a.depth = ctx->max_depth;
+    int units = std::max(ctx->n_tail + ctx->n_coarsest, (ctx->n_res_tiles + 7) / 8);
+    for (int L = 0; L < a.depth; ++L) {
+        a.tiles[L] = ctx->d_ft_tiles[L];
+        a.n_tiles[L] = ctx->n_ft_tiles[L];
+        a.small[L] = ctx->ft_small[L];
+        units = std::max(units, a.n_tiles[L]);
     }
-    ctx->cycle_launches = ctx->launches - l0;
-    ctx->launches = l0;
-    ctx->stream = s;
-    cudaGraph_t out = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(ctx->body_stream, &out);
-    if (r != LBFS_OK) return r;
-    if (e2 != cudaSuccess) return fail(ctx, LBFS_ECUDA, std::string("cycle body capture: ") + cudaGetErrorString(e2));
-    return LBFS_OK;
+    a.tail = ctx->d_tail;
+    a.coarsest = ctx->d_coarsest;
+    a.n_tail = ctx->n_tail;
+    a.n_coarsest = ctx->n_coarsest;
+    a.tail_cells = ctx->tail_cells;
+    a.tail_small = ctx->tail_small;
+    a.strips = ctx->d_res_tiles;
+    a.n_strips = ctx->n_res_tiles;
+    a.rows = ctx->res_rows;
+    return launch_mg_cycles(ctx->prec, a, std::min(units, ctx->sm_count), ctx->n_coarsest > 0 ? ctx->coarsest_cells : 0,
+                            pot_check(ctx, 0, kmax, nullptr), ctx->stream);
 }
 
-// The warm potential solve as a graph of its own, launched by eager steps.
-lbfs_status build_pot_graph(lbfs_ctx* ctx) {
-    if (!ctx->cap_stream) CK(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-    cudaStream_t user = ctx->stream;
-    const int64_t l0 = ctx->launches;
-    ctx->stream = ctx->cap_stream;
-    ctx->capturing = true;
-    cudaError_t e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal);
-    lbfs_status r = e == cudaSuccess ? capture_warm_potential(ctx) : LBFS_ECUDA;
-    cudaGraph_t g = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &g);
-    ctx->capturing = false;
-    ctx->stream = user;
-    ctx->launches = l0;
-    if (e != cudaSuccess) return fail(ctx, LBFS_ECUDA, std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e));
-    if (r != LBFS_OK) {
-        if (g) cudaGraphDestroy(g);
-        return r;
-    }
-    if (e2 != cudaSuccess) return fail(ctx, LBFS_ECUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e2));
-    ctx->pot_graph = g;
-    CK(cudaGraphInstantiate(&ctx->pot_exec, g, 0));
-    return LBFS_OK;
+// Cycles launched phase by phase before the kernel that runs as many as are still needed; what is
+// launched for a converged case returns at once.  A grid barrier costs more than a launch of a
+// recorded graph (a cycle on 128 x 64 takes 46 us by launches, 57 in one kernel), so the first
+// cycles of a step that is likely to need them are launched: four in FP64, whose warm steps take
+// three to six (3 to 6 launched are within 3%), and one in a batch of at least four cases, of which
+// one needs a cycle in every other step (64 cases: 780 us a step against 911; 4: 150 against 166).
+// A single mixed case mostly takes none, for which the one kernel alone is the cheaper: 5 us, against
+// 16 for a conditional graph node (512 x 256: 89 us a step, 93 with a launched cycle).
+int phased_cycles(int prec, int cases) {
+    return prec == 0 ? 4 : (cases >= 4 ? 1 : 0);
 }
 
-// The potential of the current state.
-// After a state is set (pot_fresh), refinement cycles run until every case meets
-// mg_tol, checked on the host after each cycle (at most mg_max_cycles).
-// Every later step is the warm solve above (no host round trip): inline in a recorded
-// step graph, or its own graph launched by an eager step.  A case still above mg_tol
-// after mg_warm_cycles cycles is marked as failed (LBFS_ENOTCONVERGED at the end of
-// lbfs_step).  So the reported residual is always that of the potential the
-// thermo-fluid stages use.
+// The potential of the current state: in FP64 a warm step starts from the linearly
+// extrapolated potential; then the step's first residual and check, then refinement cycles
+// (V-cycle, correction, residual of the corrected potential, check), which the checks end on the
+// device, so a step whose start already meets mg_tol runs none and no host round trip is
+// made.  At most mg_warm_cycles cycles, or mg_max_cycles after a state was set (pot_fresh); a
+// case still above mg_tol then is marked as failed (LBFS_ENOTCONVERGED at the end of lbfs_step).
+// So the reported residual is always that of the potential the thermo-fluid stages use.
 lbfs_status potential_solve(lbfs_ctx* ctx) {
     if (ctx->n_pot == 0) return LBFS_OK;
-    const int p = ctx->prec;
+    const int kmax = ctx->pot_fresh ? ctx->mg_max_cycles : ctx->mg_warm_cycles;
     cudaStream_t s = ctx->stream;
-    if (!ctx->pot_fresh && ctx->cfg.mg_plain_cycles) {
-        // the same cycles as plain launches; each kernel returns at once for a converged case
-        const int K = ctx->mg_warm_cycles;
-        int* nd = ctx->d_flag + 1;
-        if (p == 0) LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
-        LK(check_residual(ctx, 1, K, nd, nullptr, 0, 0));
-        for (int c = 0; c < K; ++c) {
+    if (ctx->prec == 0 && !ctx->pot_fresh)
+        LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
+    if (ctx->cfg.mg_plain_cycles && ctx->pot_fresh) {   // as many as are needed, counted on the host
+        for (int it = 0;; ++it) {
+            CK(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s));
+            LK(check_residual(ctx, it == 0, kmax, ctx->d_flag));
+            CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            if (*ctx->h_flag == 0) break;
             lbfs_status r = vcycle(ctx);
             if (r != LBFS_OK) return r;
-            LK(check_residual(ctx, 0, K, nd, nullptr, 0, 0));
         }
-        CK(cudaMemsetAsync(nd, 0, sizeof(int), s));
-        return LBFS_OK;
-    }
-    if (!ctx->pot_fresh) {
-        if (ctx->capturing) return capture_warm_potential(ctx);
-        if (!ctx->pot_exec) {
-            lbfs_status r = build_pot_graph(ctx);
+    } else {
+        const int phased = ctx->cfg.mg_plain_cycles ? kmax : std::min(kmax, phased_cycles(ctx->prec, ctx->n_pot));
+        LK(check_residual(ctx, 1, kmax, nullptr));
+        for (int c = 0; c < phased; ++c) {
+            lbfs_status r = vcycle(ctx);
             if (r != LBFS_OK) return r;
+            LK(check_residual(ctx, 0, kmax, nullptr));
         }
-        CK(cudaGraphLaunch(ctx->pot_exec, s));
-        ctx->launches += p == 0 ? 2 : 1;   // (FP64: the extrapolated start) residual with its check
-        return LBFS_OK;
+        if (phased < kmax) LK(cycles(ctx, kmax));
     }
-    for (int it = 0;; ++it) {
-        CK(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s));
-        LK(check_residual(ctx, it == 0, 1 << 30, ctx->d_flag, nullptr, 0, 0));
-        CK(cudaMemcpyAsync(ctx->h_flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        if (*ctx->h_flag == 0) break;
-        if (it == ctx->mg_max_cycles) {
-            ctx->pot_fail = true;
-            break;
-        }
-        lbfs_status r = vcycle(ctx);
-        if (r != LBFS_OK) return r;
+    if (ctx->pot_fresh) {
+        // the warm steps that follow extrapolate only once they have stored a potential
+        for (size_t c = 0; c < ctx->slots.size(); ++c)
+            if (ctx->slots[c].defined)
+                CK(cudaMemsetAsync(ctx->d_stats + c * kStatN + ST_EXTRAP, 0, sizeof(double), s));
+        ctx->pot_fresh = false;
     }
-    // the warm steps that follow extrapolate only once they have stored a potential
-    for (size_t c = 0; c < ctx->slots.size(); ++c)
-        if (ctx->slots[c].defined) CK(cudaMemsetAsync(ctx->d_stats + c * kStatN + ST_EXTRAP, 0, sizeof(double), s));
-    ctx->pot_fresh = false;
     return LBFS_OK;
 }
 
@@ -747,7 +686,7 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
         lbfs_destroy(ctx);
         return LBFS_ENOMEM;
     }
-    cudaMemset(ctx->d_cases, 0, cases_b + stage_b + stats_b + 256);   // d_flag: [0] host-checked votes, [1] device votes, [2] ticket
+    cudaMemset(ctx->d_cases, 0, cases_b + stage_b + stats_b + 256);   // d_flag: [0] host-checked votes, [1] and [2] the cycles' grid barrier
     if (cudaDeviceSynchronize() != cudaSuccess) {
         lbfs_destroy(ctx);
         return LBFS_ECUDA;
@@ -836,6 +775,7 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
         add(&hd.lev[L].mu, lc * (L == 0 ? rs : sizeof(float)));
         add(&hd.lev[L].e, lc * sizeof(float));
         add(&hd.lev[L].r, lc * (L == 0 ? rs : sizeof(float)));
+        if (L > 0 && L < hd.tail) add(&hd.lev[L].eu, lc * sizeof(float));
     }
     const int red_groups = (red_cap + kStageGroup - 1) / kStageGroup;
     add((void**)&hd.red, (size_t)red_cap * kRedN * sizeof(double));
@@ -853,6 +793,8 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     s.block = dalloc(ctx, off);
     if (!s.block) return fail(ctx, LBFS_ENOMEM, "device allocation of the case failed");
     for (auto& pr : plan) *pr.first = static_cast<char*>(s.block) + pr.second;
+    for (int L = 0; L < nlev; ++L)
+        if (!hd.lev[L].eu) hd.lev[L].eu = hd.lev[L].e;
     if (ctx->prec == 0) hd.phi = hd.phi64;
     hd.stats = ctx->d_stats + (size_t)id * kStatN;
     s.hd = hd;
@@ -1019,13 +961,6 @@ lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
     CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, nb, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     harvest(ctx);
-    if (ctx->n_pot > 0 && ctx->cycle_launches > 0 && !ctx->cfg.mg_plain_cycles) {
-        // refinement cycles run by device-decided loops: at least the most any case ran
-        double cyc = 0.0;
-        for (size_t c = 0; c < ctx->slots.size(); ++c)
-            if (ctx->slots[c].defined) cyc = std::fmax(cyc, ctx->h_stats[c * kStatN + ST_POT_CYCLES_SUM]);
-        ctx->launches += (int64_t)cyc * ctx->cycle_launches;
-    }
     bool bad = false;
     for (size_t c = 0; c < ctx->slots.size(); ++c) {
         const double* st = ctx->h_stats + c * kStatN;
@@ -1130,7 +1065,6 @@ void lbfs_destroy(lbfs_ctx* ctx) {
     harvest(ctx);
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-    if (ctx->body_stream) cudaStreamDestroy(ctx->body_stream);
     for (Slot& s : ctx->slots) free_slot(ctx, s);
     for (auto* p : ctx->d_ft_tiles) dfree(ctx, p);
     dfree(ctx, ctx->d_mg_tiles);

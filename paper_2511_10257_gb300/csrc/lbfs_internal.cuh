@@ -76,7 +76,9 @@ struct MGLevel {
     float wlx, wly;
     int ragged;  // wlx < 1 or wly < 1
     void* mu;   // cell coefficient mu_m (FP32; FP64 on the fine level of the FP64 mode)
-    void* e;    // correction (FP32)
+    void* e;    // correction (FP32), pre-smoothed
+    void* eu;   // the finished correction of a coarse level: an array of its own where a kernel leg writes it
+                // (tiles read their neighbours' e), e where one block holds the whole level
     void* r;    // right-hand side / residual (as mu)
 };
 

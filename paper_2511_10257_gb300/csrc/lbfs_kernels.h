@@ -27,19 +27,15 @@ constexpr int kMgTX = 32, kMgTY = 32;
 // The residual takes strips of kResidStripW columns by `rows` rows, one warp each, and checks
 // each case once its strips are done.  first: the step's first residual (every case; later ones
 // skip converged cases).  tol: the convergence test.  A case still above tol gets another cycle
-// (one more vote in not_done) unless it has had kmax, when it is marked as failed.  set_cond:
-// the call runs inside a conditional graph node; the last of ncases to decide (ticket) sets cond
-// to 1 while a case needs another cycle.
+// (one more vote in not_done, if given) unless it has had kmax, when it is marked as failed.
+// sync: the grid barrier of launch_mg_cycles (two counters), cleared by a first check.
 constexpr int kResidStripW = 30, kResidMinRows = 2;
 struct PotCheck {
     int first;
     double tol;
     int kmax;
     int* not_done;
-    unsigned* ticket;
-    int ncases;
-    cudaGraphConditionalHandle cond;
-    int set_cond;
+    unsigned* sync;
 };
 cudaError_t launch_mg_residual(int prec, const DevCase* cases, const TileRef* tiles, int n, int rows, const PotCheck& ck,
                                cudaStream_t st);
@@ -64,6 +60,21 @@ cudaError_t launch_mg_vdown(int prec, const DevCase* cases, const TileRef* tiles
                             cudaStream_t st);
 cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, int n, int level, int small,
                           cudaStream_t st);
+// Cycles (V-cycle, residual, check) until no case needs another, in one cooperative launch of
+// `blocks` blocks (at most one an SM), after a first launch_mg_residual with the same check
+// and first set to 0.  max_coarsest: as for launch_mg_coarsest, 0 without such a case.
+struct CycleArgs {
+    const DevCase* cases;
+    const TileRef* tiles[kMaxLevels];   // of the fused legs, per level with a kernel per leg
+    int n_tiles[kMaxLevels], small[kMaxLevels];
+    int depth;
+    const int *tail, *coarsest;         // cases by how their coarse levels are solved
+    int n_tail, n_coarsest, tail_cells, tail_small;
+    const TileRef* strips;              // of the residual
+    int n_strips, rows;
+};
+cudaError_t launch_mg_cycles(int prec, const CycleArgs& a, int blocks, int max_coarsest, const PotCheck& ck,
+                             cudaStream_t st);
 
 // per-case utility kernels (lbfs_fields.cu)
 struct InitArgs {

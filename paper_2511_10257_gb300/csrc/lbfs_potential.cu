@@ -20,6 +20,7 @@
 // carry the true face length over centre distance, and the prolongation interpolates
 // between the true centres, so every grid size keeps the contraction of the even
 // ones.
+#include <algorithm>
 #include <type_traits>
 
 #include "lbfs_kernels.h"
@@ -250,24 +251,6 @@ __device__ __forceinline__ FaceTerm<float> face_terms(const PotCell<float>& c, c
 __device__ __forceinline__ double shfl_right(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ float shfl_right(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
-// The one call of cudaGraphSetConditional of a check: every case adds one to the ticket
-// after it has added its vote to not_done; the last one sets the loop condition (run
-// another cycle while a case still needs one) and clears both counters.
-__device__ __forceinline__ void decide_next_cycle(int* not_done, unsigned* ticket, int ncases,
-                                                  cudaGraphConditionalHandle cond) {
-    if (ncases == 1) {   // the only case is done (decide() handles one that is not)
-        cudaGraphSetConditional(cond, 0u);
-        return;
-    }
-    __threadfence();
-    if (atomicAdd(ticket, 1u) == (unsigned)(ncases - 1)) {
-        __threadfence();
-        const int nd = atomicExch(not_done, 0);
-        *ticket = 0u;
-        cudaGraphSetConditional(cond, nd > 0 ? 1u : 0u);
-    }
-}
-
 // The relative residual of a case is known: converged, failed, or one cycle more.  A case that
 // has not converged gets another cycle unless it has had kmax, in which case it is marked as
 // failed and left alone.  first: the step's first check (resets the cycle count).
@@ -278,6 +261,7 @@ __device__ __forceinline__ void decide(const DevCase* dc, const PotCheck& ck, do
     if (ck.first) {
         st[ST_POT_CYCLES] = 0.0;
         st[ST_EXTRAP] = 1.0;   // from now on phi_prev holds a step's potential (FP64)
+        ck.sync[0] = ck.sync[1] = 0u;   // the grid barrier of the cycles that may follow
     }
     if (rel <= ck.tol) {
         st[ST_POT_DONE] = 1.0;
@@ -293,13 +277,8 @@ __device__ __forceinline__ void decide(const DevCase* dc, const PotCheck& ck, do
             if (rms > 0.0 && isfinite(rms)) frexp(rms, &ex);
             st[ST_SCALE] = ldexp(1.0, ex < -1000 ? 1000 : -ex);
         }
-        if (ck.set_cond && ck.ncases == 1) {
-            cudaGraphSetConditional(ck.cond, 1u);
-            return;
-        }
-        atomicAdd(ck.not_done, 1);
+        if (ck.not_done) atomicAdd(ck.not_done, 1);
     }
-    if (ck.set_cond) decide_next_cycle(ck.not_done, ck.ticket, ck.ncases, ck.cond);
 }
 
 // One warp per strip of kResidW columns and `rows` rows, one lane per column and one halo
@@ -310,16 +289,10 @@ __device__ __forceinline__ void decide(const DevCase* dc, const PotCheck& ck, do
 constexpr int kResidW = kResidStripW;
 
 template <class M>
-__global__ void __launch_bounds__(32) k_residual(const DevCase* __restrict__ cases, const TileRef* __restrict__ tiles,
-                                                 int rows, const PotCheck ck) {
+__device__ __forceinline__ void residual_strip(const DevCase* __restrict__ dc, const TileRef tr, int rows,
+                                               const PotCheck& ck, int lane) {
     using Slot = typename DSum<M>::Slot;
-    const TileRef tr = tiles[blockIdx.x];
-    const DevCase* dc = cases + tr.case_id;
-    const int lane = threadIdx.x;
-    if (!ck.first && pot_done(dc)) {
-        if (ck.set_cond && tr.slot == 0 && lane == 0) decide_next_cycle(ck.not_done, ck.ticket, ck.ncases, ck.cond);
-        return;
-    }
+    if (!ck.first && pot_done(dc)) return;
     const CaseParams& P = dc->P;
     const int nx = P.nx, ny = P.ny;
     const unsigned pitch = (unsigned)P.pitch;
@@ -455,6 +428,13 @@ __global__ void __launch_bounds__(32) k_residual(const DevCase* __restrict__ cas
     if (lane != 0) return;
     if (ck.first) dc->stats[ST_B2] = b2.value();
     decide(dc, ck, r2.value(), ck.first ? b2.value() : dc->stats[ST_B2], sizeof(M) == 8);
+}
+
+template <class M>
+__global__ void __launch_bounds__(32) k_residual(const DevCase* __restrict__ cases, const TileRef* __restrict__ tiles,
+                                                 int rows, const PotCheck ck) {
+    const TileRef tr = tiles[blockIdx.x];
+    residual_strip<M>(cases + tr.case_id, tr, rows, ck, threadIdx.x);
 }
 
 // A case's walls as one word held in a register: bits 0-3 Dirichlet walls, 4 and 5 periodic axes.
@@ -611,11 +591,11 @@ __device__ __forceinline__ M region_apply(int dirichlet, const MGLevel& lv, int 
 template <class M, int TX, int TY, int H>
 __device__ __forceinline__ void region_half_sweep(int dirichlet, const MGLevel& lv, int x0, int y0,
                                                   const M* mu, const M* r, M* e, const unsigned char* in, int c,
-                                                  int h) {
+                                                  int h, int tid, int nt) {
     using G = FRegion<TX, TY, H>;
     const int VW = G::W - 2 * h, VH = G::Hh - 2 * h, HW = (VW + 1) / 2;
     const int base = (x0 - H) + (y0 - H);
-    for (int t = threadIdx.x; t < HW * VH; t += blockDim.x) {
+    for (int t = tid; t < HW * VH; t += nt) {
         const int ly = h + t / HW;
         const int lx = h + ((c - base - ly - h) & 1) + 2 * (t % HW);
         if (lx >= G::W - h) continue;
@@ -629,12 +609,13 @@ __device__ __forceinline__ void region_half_sweep(int dirichlet, const MGLevel& 
 
 template <class S, class M, int TX, int TY, int H>
 __device__ __forceinline__ void region_load(const CaseParams& P, const MGLevel& lv, int x0, int y0, M* smu,
-                                            M* sr, M* se, unsigned char* in, bool load_e, S scale) {
+                                            M* sr, M* se, unsigned char* in, bool load_e, S scale, int tid,
+                                            int nt) {
     using G = FRegion<TX, TY, H>;
     const S* mu = static_cast<const S*>(lv.mu);
     const S* r = static_cast<const S*>(lv.r);
     const M* e = static_cast<const M*>(lv.e);
-    for (int k = threadIdx.x; k < G::N; k += blockDim.x) {
+    for (int k = tid; k < G::N; k += nt) {
         int gx, gy, sx, sy;
         const int ok = region_source(P, lv.nx, lv.ny, x0, y0, H, G::W, k, gx, gy, sx, sy);
         const unsigned g = (unsigned)sy * (unsigned)lv.pitch + (unsigned)sx;
@@ -647,28 +628,30 @@ __device__ __forceinline__ void region_load(const CaseParams& P, const MGLevel& 
 
 // S: the type in which the level keeps mu and r (double on the fine level of the FP64 mode,
 // whose residual enters scaled); everything else is FP32.
-template <class S, int TX, int TY>
-__global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases,
-                                               const TileRef* __restrict__ tiles, int L) {
+// The tile's nt threads (tid: this one) meet at sync(); mem: kLegBytes<TX, TY> bytes of shared memory.
+template <int TX, int TY>
+constexpr int kLegBytes = (13 * FRegion<TX, TY, kHD>::N + 15) / 16 * 16;
+
+template <class S, int TX, int TY, class Sync>
+__device__ __forceinline__ void vdown_tile(const DevCase* __restrict__ dc, const TileRef tr, int L, unsigned char* mem,
+                                           int tid, int nt, Sync sync) {
     using M = float;
     using G = FRegion<TX, TY, kHD>;
-    __shared__ M smu[G::N], sr[G::N], se[G::N];
-    __shared__ unsigned char in[G::N];
-    const TileRef tr = tiles[blockIdx.x];
-    const DevCase* dc = cases + tr.case_id;
+    M *smu = reinterpret_cast<M*>(mem), *sr = smu + G::N, *se = sr + G::N;
+    unsigned char* in = reinterpret_cast<unsigned char*>(se + G::N);
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
     const int dirichlet = wall_mask(P);
     const MGLevel lv = dc->lev[L], cv = dc->lev[L + 1];
-    region_load<S, M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, sr, se, in, false, pot_scale<S>(dc));
-    __syncthreads();
+    region_load<S, M, TX, TY, kHD>(P, lv, tr.x0, tr.y0, smu, sr, se, in, false, pot_scale<S>(dc), tid, nt);
+    sync();
     for (int h = 1; h <= 2 * kFNu; ++h) {
-        region_half_sweep<M, TX, TY, kHD>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
-        __syncthreads();
+        region_half_sweep<M, TX, TY, kHD>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h, tid, nt);
+        sync();
     }
     // pre-smoothed correction of the tile
     M* e = static_cast<M*>(lv.e);
-    for (int t = threadIdx.x; t < TX * TY; t += blockDim.x) {
+    for (int t = tid; t < TX * TY; t += nt) {
         const int gx = tr.x0 + t % TX, gy = tr.y0 + t / TX;
         if (gx < lv.nx && gy < lv.ny)
             e[(unsigned)gy * (unsigned)lv.pitch + (unsigned)gx] = se[(t / TX + kHD) * G::W + t % TX + kHD];
@@ -678,7 +661,7 @@ __global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases
     // the coarse coefficient as the mean of the children's
     M* rc = static_cast<M*>(cv.r);
     M* muc = static_cast<M*>(cv.mu);
-    for (int t = threadIdx.x; t < (TX / 2) * (TY / 2); t += blockDim.x) {
+    for (int t = tid; t < (TX / 2) * (TY / 2); t += nt) {
         const int ci = t % (TX / 2), cj = t / (TX / 2);
         const int I = tr.x0 / 2 + ci, J = tr.y0 / 2 + cj;
         if (I >= cv.nx || J >= cv.ny) continue;
@@ -709,27 +692,25 @@ __global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases
 
 // FINE: the fine level, where the smoothed correction goes straight into the master potential
 // (M0: its precision) instead of back to e.
-template <class S, class M0, bool FINE, int TX, int TY>
-__global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
-                                             const TileRef* __restrict__ tiles, int L) {
+template <class S, class M0, bool FINE, int TX, int TY, class Sync>
+__device__ __forceinline__ void vup_tile(const DevCase* __restrict__ dc, const TileRef tr, int L, unsigned char* mem,
+                                         int tid, int nt, Sync sync) {
     using M = float;
     using G = FRegion<TX, TY, kHU>;
     constexpr int CW = (TX + 2 * kHU) / 2 + 3, CH = (TY + 2 * kHU) / 2 + 3;
-    __shared__ M smu[G::N], sr[G::N], se[G::N];
-    __shared__ M sc[CW * CH];
-    __shared__ unsigned char in[G::N];
-    const TileRef tr = tiles[blockIdx.x];
-    const DevCase* dc = cases + tr.case_id;
+    static_assert(13 * G::N + 4 * CW * CH <= kLegBytes<TX, TY>, "the up leg fits the down leg's memory");
+    M *smu = reinterpret_cast<M*>(mem), *sr = smu + G::N, *se = sr + G::N, *sc = se + G::N;
+    unsigned char* in = reinterpret_cast<unsigned char*>(sc + CW * CH);
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
     const int dirichlet = wall_mask(P);
     const MGLevel lv = dc->lev[L], cv = dc->lev[L + 1];
-    region_load<S, M, TX, TY, kHU>(P, lv, tr.x0, tr.y0, smu, sr, se, in, true, pot_scale<S>(dc));
+    region_load<S, M, TX, TY, kHU>(P, lv, tr.x0, tr.y0, smu, sr, se, in, true, pot_scale<S>(dc), tid, nt);
     // coarse corrections around the region (one cell beyond its parents)
     const int cx0 = (tr.x0 - kHU) / 2 - 1 - ((tr.x0 - kHU) < 0 ? 1 : 0);
     const int cy0 = (tr.y0 - kHU) / 2 - 1 - ((tr.y0 - kHU) < 0 ? 1 : 0);
-    const M* ec = static_cast<const M*>(cv.e);
-    for (int k = threadIdx.x; k < CW * CH; k += blockDim.x) {
+    const M* ec = static_cast<const M*>(cv.eu);
+    for (int k = tid; k < CW * CH; k += nt) {
         int I = cx0 + k % CW, J = cy0 + k / CW;
         // periodic axes wrap; across a wall only the one-cell ghost is ever used by a
         // cell inside the domain, so the rest is clamped onto it
@@ -739,8 +720,8 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
         else J = J < -1 ? -1 : (J > cv.ny ? cv.ny : J);
         sc[k] = coarse_at<M>(dirichlet, ec, cv.nx, cv.ny, cv.pitch, I, J);
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < G::N; k += blockDim.x) {
+    sync();
+    for (int k = tid; k < G::N; k += nt) {
         if (!in[k]) continue;
         const int gx = tr.x0 - kHU + k % G::W, gy = tr.y0 - kHU + k / G::W;
         // parent of the region cell in unwrapped level coordinates
@@ -761,13 +742,13 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
         }
         se[k] += v;
     }
-    __syncthreads();
+    sync();
     for (int h = 1; h <= 2 * kFNu; ++h) {
-        region_half_sweep<M, TX, TY, kHU>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h);
-        __syncthreads();
+        region_half_sweep<M, TX, TY, kHU>(dirichlet, lv, tr.x0, tr.y0, smu, sr, se, in, (h - 1) & 1, h, tid, nt);
+        sync();
     }
-    M* e = static_cast<M*>(lv.e);
-    for (int t = threadIdx.x; t < TX * TY; t += blockDim.x) {
+    M* e = static_cast<M*>(lv.eu);
+    for (int t = tid; t < TX * TY; t += nt) {
         const int gx = tr.x0 + t % TX, gy = tr.y0 + t / TX;
         if (gx < lv.nx && gy < lv.ny) {
             const unsigned k = (unsigned)gy * (unsigned)lv.pitch + (unsigned)gx;
@@ -778,15 +759,29 @@ __global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
     }
 }
 
+template <class S, int TX, int TY>
+__global__ void __launch_bounds__(256) k_vdown(const DevCase* __restrict__ cases,
+                                               const TileRef* __restrict__ tiles, int L) {
+    __shared__ __align__(16) unsigned char mem[kLegBytes<TX, TY>];
+    const TileRef tr = tiles[blockIdx.x];
+    vdown_tile<S, TX, TY>(cases + tr.case_id, tr, L, mem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+}
+
+template <class S, class M0, bool FINE, int TX, int TY>
+__global__ void __launch_bounds__(256) k_vup(const DevCase* __restrict__ cases,
+                                             const TileRef* __restrict__ tiles, int L) {
+    __shared__ __align__(16) unsigned char mem[kLegBytes<TX, TY>];
+    const TileRef tr = tiles[blockIdx.x];
+    vup_tile<S, M0, FINE, TX, TY>(cases + tr.case_id, tr, L, mem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+}
+
+constexpr int kTailNT = 1024;   // threads of the kernels that take a case's coarse levels, and of the cycles
+
 // conjugate gradients on the coarsest level, one block per case, in shared memory
 // (for coarsest levels too large for the tail kernel: a periodic axis that halves to an odd
 // size early)
-__global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ cases,
-                                                  const int* __restrict__ ids) {
+__device__ __forceinline__ void coarsest_case(const DevCase* __restrict__ dc, unsigned char* smem_raw, float* red) {
     using M = float;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ M red[32];
-    const DevCase* dc = cases + ids[blockIdx.x];
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
     const MGLevel lv = dc->lev[dc->nlev - 1];
@@ -840,6 +835,12 @@ __global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ ca
     }
 }
 
+__global__ void __launch_bounds__(kTailNT) k_coarsest(const DevCase* __restrict__ cases, const int* __restrict__ ids) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float red[32];
+    coarsest_case(cases + ids[blockIdx.x], smem_raw, red);
+}
+
 // ---- the coarse levels in one kernel ---------------------------------------------------
 // One block per case takes the V-cycle from level dc->tail (at most kTailCells cells) down to
 // the coarsest level and back, all in shared memory: on small levels a kernel per leg is all
@@ -851,7 +852,7 @@ __global__ void __launch_bounds__(256) k_coarsest(const DevCase* __restrict__ ca
 // takes the block's first kTailFew threads and runs twice, so that it stands for an exact solve: with one pass the potential's error at the
 // same residual is half as large again.  A case whose tail starts at
 // level 0 adds the correction to its potential here.
-constexpr int kTailNT = 1024, kTailFew = 256, kTailPasses = 2, kTinyCells = 16;
+constexpr int kTailFew = 256, kTailPasses = 2, kTinyCells = 16;
 
 struct TailLevel {
     int nx, ny, off, ragged;   // off: of its cells in the arrays below
@@ -885,12 +886,8 @@ __device__ __forceinline__ void tail_sync(int nt) {
 }
 
 template <class M0>
-__global__ void __launch_bounds__(kTailNT) k_tail(const DevCase* __restrict__ cases, const int* __restrict__ ids,
-                                                  int max_cells, int max_small) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ TailLevel lv[kMaxLevels];
-    __shared__ MGLevel geo[kMaxLevels];
-    const DevCase* dc = cases + ids[blockIdx.x];
+__device__ __forceinline__ void tail_case(const DevCase* __restrict__ dc, int max_cells, int max_small,
+                                          unsigned char* smem_raw, TailLevel* lv, MGLevel* geo) {
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
     const int L0 = dc->tail, n_lev = dc->nlev - L0;
@@ -1188,6 +1185,121 @@ __global__ void __launch_bounds__(kTailNT) k_tail(const DevCase* __restrict__ ca
     });
 }
 
+template <class M0>
+__global__ void __launch_bounds__(kTailNT) k_tail(const DevCase* __restrict__ cases, const int* __restrict__ ids,
+                                                  int max_cells, int max_small) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ TailLevel lv[kMaxLevels];
+    __shared__ MGLevel geo[kMaxLevels];
+    tail_case<M0>(cases + ids[blockIdx.x], max_cells, max_small, smem_raw, lv, geo);
+}
+
+// ---- refinement cycles until every case has converged, in one cooperative kernel --------
+// The kernels above as phases of one grid, a block an SM, with a grid barrier between
+// dependent phases: a leg's tile takes kLegNT threads, a coarse solve a block, a residual strip
+// a warp.  When the check before it found every case converged the kernel returns at once.
+// The phases run the same code on the same data as the kernels of their own: the potential is
+// the same bit for bit.
+constexpr int kLegNT = 256, kLegGroups = kTailNT / kLegNT;
+
+// All blocks of the grid arrive (sync[0] counts them; it starts a launch at zero and only
+// grows).  The blocks of a cooperative launch run at the same time, so the wait ends; should it
+// not within kSyncPolls polls (seconds), sync[1] tells every block to give up.
+constexpr int kSyncPolls = 1 << 22;
+
+__device__ __forceinline__ bool grid_sync(unsigned* sync, unsigned& target, int* ok) {
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(sync, 1u);
+        int polls = 0;
+        while (*static_cast<volatile unsigned*>(sync) < target && ++polls < kSyncPolls &&
+               *static_cast<volatile unsigned*>(sync + 1) == 0u) {
+        }
+        __threadfence();
+        *ok = *static_cast<volatile unsigned*>(sync) >= target;
+        if (!*ok) atomicExch(sync + 1, 1u);
+    }
+    __syncthreads();
+    return *ok != 0;
+}
+
+template <class M0>
+__global__ void __launch_bounds__(kTailNT, 1) k_cycles(const __grid_constant__ CycleArgs a, const PotCheck ck) {
+    extern __shared__ __align__(16) unsigned char mem[];
+    __shared__ TailLevel lv[kMaxLevels];
+    __shared__ MGLevel geo[kMaxLevels];
+    __shared__ float red[32];
+    __shared__ int ok;
+    const int nb = gridDim.x, b = blockIdx.x, cases_n = a.n_tail + a.n_coarsest;
+    auto case_of = [&](int q) { return a.cases + (q < a.n_tail ? a.tail[q] : a.coarsest[q - a.n_tail]); };
+    auto pending = [&] {   // does a case still need a cycle?
+        int n = 0;
+        for (int q = threadIdx.x; q < cases_n; q += kTailNT) n |= !pot_done(case_of(q));
+        return __syncthreads_or(n) != 0;
+    };
+    if (!pending()) return;
+    unsigned target = 0;
+    const int group = threadIdx.x / kLegNT, tid = threadIdx.x % kLegNT;
+    auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(2 + group), "n"(kLegNT) : "memory"); };
+    unsigned char* const leg = mem + group * kLegBytes<kFusedTX, kFusedTY>;
+    bool more;
+    do {
+        bool alive = true;
+        for (int L = 0; L < a.depth && alive; ++L) {
+            for (int t = group * nb + b; t < a.n_tiles[L]; t += kLegGroups * nb) {
+                const TileRef tr = a.tiles[L][t];
+                const DevCase* dc = a.cases + tr.case_id;
+                const bool wide = sizeof(M0) == 8 && L == 0;
+                if (a.small[L]) {
+                    if (wide) vdown_tile<M0, kFusedSmallTX, kFusedSmallTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                    else vdown_tile<float, kFusedSmallTX, kFusedSmallTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                } else {
+                    if (wide) vdown_tile<M0, kFusedTX, kFusedTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                    else vdown_tile<float, kFusedTX, kFusedTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                }
+                sync();   // the tile's memory is free again
+            }
+            alive = grid_sync(ck.sync, target, &ok);
+        }
+        for (int q = b; q < cases_n && alive; q += nb) {
+            if (q < a.n_tail) tail_case<M0>(case_of(q), a.tail_cells, a.tail_small, mem, lv, geo);
+            else coarsest_case(case_of(q), mem, red);
+            __syncthreads();
+        }
+        alive = alive && grid_sync(ck.sync, target, &ok);
+        for (int L = a.depth - 1; L >= 0 && alive; --L) {
+            for (int t = group * nb + b; t < a.n_tiles[L]; t += kLegGroups * nb) {
+                const TileRef tr = a.tiles[L][t];
+                const DevCase* dc = a.cases + tr.case_id;
+                if (L > 0) {
+                    if (a.small[L]) vup_tile<float, float, false, kFusedSmallTX, kFusedSmallTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                    else vup_tile<float, float, false, kFusedTX, kFusedTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                } else {
+                    if (a.small[L]) vup_tile<M0, M0, true, kFusedSmallTX, kFusedSmallTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                    else vup_tile<M0, M0, true, kFusedTX, kFusedTY>(dc, tr, L, leg, tid, kLegNT, sync);
+                }
+                sync();
+            }
+            alive = grid_sync(ck.sync, target, &ok);
+        }
+        if (alive) {
+            for (int t = (threadIdx.x >> 5) * nb + b; t < a.n_strips; t += (kTailNT >> 5) * nb) {
+                const TileRef tr = a.strips[t];
+                residual_strip<M0>(a.cases + tr.case_id, tr, a.rows, ck, threadIdx.x & 31);
+            }
+            alive = grid_sync(ck.sync, target, &ok);
+        }
+        if (!alive) {   // reported as a potential that has not converged
+            for (int q = threadIdx.x; q < cases_n; q += kTailNT)
+                if (!pot_done(case_of(q))) case_of(q)->stats[ST_POT_FAIL] = 1.0;
+            return;
+        }
+        more = pending();
+    } while (more);
+}
+
 // The FP64 warm start, extrapolated linearly in time: phi <- 2 phi - phi_prev and
 // phi_prev <- phi, cell by cell, once phi_prev holds the previous step's potential
 // (ST_EXTRAP set); before that phi_prev <- phi only.  A start closer to the step's
@@ -1364,10 +1476,14 @@ cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, 
     return cudaGetLastError();
 }
 
+static size_t tail_bytes(int max_cells, int max_small) {
+    return (size_t)6 * max_cells * sizeof(float) + (size_t)max_small * (2 * sizeof(float) + 6 * sizeof(short));
+}
+
 cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* ids, int ncases, int max_cells, int max_small,
                            cudaStream_t st) {
     if (ncases <= 0) return cudaSuccess;
-    const size_t sm = (size_t)6 * max_cells * sizeof(float) + (size_t)max_small * (2 * sizeof(float) + 6 * sizeof(short));
+    const size_t sm = tail_bytes(max_cells, max_small);
     auto kern = prec == 0 ? k_tail<double> : k_tail<float>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1380,8 +1496,19 @@ cudaError_t launch_mg_coarsest(const DevCase* cases, const int* ids, int ncases,
     const size_t sm = (size_t)5 * max_cells * sizeof(float);
     const cudaError_t e = cudaFuncSetAttribute(k_coarsest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_coarsest<<<ncases, 256, sm, st>>>(cases, ids);
+    k_coarsest<<<ncases, kTailNT, sm, st>>>(cases, ids);
     return cudaGetLastError();
+}
+
+cudaError_t launch_mg_cycles(int prec, const CycleArgs& a, int blocks, int max_coarsest, const PotCheck& ck,
+                             cudaStream_t st) {
+    const size_t sm = std::max({(size_t)kLegGroups * kLegBytes<kFusedTX, kFusedTY>, tail_bytes(a.tail_cells, a.tail_small),
+                                (size_t)5 * max_coarsest * sizeof(float)});
+    auto kern = prec == 0 ? k_cycles<double> : k_cycles<float>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    void* args[] = {const_cast<CycleArgs*>(&a), const_cast<PotCheck*>(&ck)};
+    return cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(kTailNT), args, sm, st);
 }
 
 cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, cudaStream_t st) {
