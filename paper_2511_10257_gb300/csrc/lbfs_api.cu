@@ -355,14 +355,9 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             if (lc.nx * lc.ny <= kTailCoarsest) {
                 tails.push_back(c);
                 int cells = 0;
-                int warp_cells = 0;
-                for (int L = s.hd.tail; L < s.hd.nlev; ++L) {
-                    const int n = s.hd.lev[L].nx * s.hd.lev[L].ny;
-                    cells += n;
-                    if (n <= kWarpCells || L == s.hd.nlev - 1) warp_cells += n;
-                }
+                for (int L = s.hd.tail; L < s.hd.nlev; ++L) cells += s.hd.lev[L].nx * s.hd.lev[L].ny;
                 tail_cells = std::max(tail_cells, cells);
-                tail_small = std::max(tail_small, warp_cells);
+                tail_small = std::max(tail_small, lc.nx * lc.ny);
             } else {
                 others.push_back(c);
                 coarsest = std::max(coarsest, lc.nx * lc.ny);

@@ -845,18 +845,23 @@ __global__ void __launch_bounds__(kTailNT) k_coarsest(const DevCase* __restrict_
 // One block per case takes the V-cycle from level dc->tail (at most kTailCells cells) down to
 // the coarsest level and back, all in shared memory: on small levels a kernel per leg is all
 // launch latency.  Red-black Gauss-Seidel sweeps, restriction and prolongation are those of the
-// fused legs; the face coefficients and the inverse diagonal are formed once per level.  Levels
-// of at most kWarpCells cells are swept by one warp, without block barriers.  The coarsest
-// level is swept 2 kFNu times when it has at most kTinyCells cells and solved by conjugate
-// gradients otherwise (grids whose one axis runs out first).  The part of at most kPassCells cells
-// takes the block's first kTailFew threads and runs twice, so that it stands for an exact solve: with one pass the potential's error at the
-// same residual is half as large again.  A case whose tail starts at
+// fused legs.  What bounds it is the chain of some 80 dependent half-sweeps, so a half-sweep is
+// kept short: cells 2t and 2t + 1 of a level, one of each colour, belong to thread t, which holds
+// their coefficients, right-hand side and neighbours' places in registers for a whole leg; only
+// the warps that own cells meet at the level's barrier, and levels of one warp need none.
+// (With every sweep reading all of it from shared memory a solve took 46.8 us on 128 x 64, each launch
+// profiled from cold caches; now 33.7.)
+// The coarsest level is swept 2 kFNu times when it has at most kTinyCells cells and solved by
+// conjugate gradients in one warp otherwise (grids whose one axis runs out first).  The part of at
+// most kPassCells cells runs twice, so that it stands for an exact solve: with one pass the
+// potential's error at the same residual is half as large again.  A case whose tail starts at
 // level 0 adds the correction to its potential here.
-constexpr int kTailFew = 256, kTailPasses = 2, kTinyCells = 16;
+constexpr int kTailPasses = 2, kTinyCells = 16;
+static_assert(kTailCells <= 2 * kTailNT, "two cells a thread on the first level");
 
 struct TailLevel {
     int nx, ny, off, ragged;   // off: of its cells in the arrays below
-    int tab;                   // of its cells in the neighbour table (levels of one warp), or -1
+    int nt;                    // threads that own cells, in whole warps
 };
 
 template <class M>
@@ -866,61 +871,58 @@ __device__ __forceinline__ M warp_allsum(M v) {
     return v;
 }
 
-// cells of a level by the first nt threads' warps, row by row: f(i, j, k), cells of one colour
-// (0, 1) or all (-1)
+// all cells of a level by the block's warps, row by row: f(i, j, k)
 template <class F>
-__device__ __forceinline__ void tail_cells(int nt, int nx, int ny, int colour, F f) {
-    const int lane = threadIdx.x & 31;
-    for (int j = threadIdx.x >> 5; j < ny; j += nt >> 5)
-        if (colour < 0) {
-            for (int i = lane; i < nx; i += 32) f(i, j, j * nx + i);
-        } else {
-            for (int i = 2 * lane + ((colour + j) & 1); i < nx; i += 64) f(i, j, j * nx + i);
-        }
+__device__ __forceinline__ void tail_cells(int nx, int ny, F f) {
+    for (int j = threadIdx.x >> 5; j < ny; j += kTailNT >> 5)
+        for (int i = threadIdx.x & 31; i < nx; i += 32) f(i, j, j * nx + i);
 }
 
-// barrier of the block, or of its first kTailFew threads
-__device__ __forceinline__ void tail_sync(int nt) {
-    if (nt == kTailNT) __syncthreads();
-    else asm volatile("bar.sync 1, %0;" ::"n"(kTailFew) : "memory");
+// places of a cell's left, right, lower and upper neighbour (the far end of the axis beyond a wall)
+__device__ __forceinline__ void tail_neighbours(int nx, int ny, int i, int j, int k, int (&n)[4]) {
+    n[0] = i > 0 ? k - 1 : k + nx - 1;
+    n[1] = i < nx - 1 ? k + 1 : k - nx + 1;
+    n[2] = j > 0 ? k - nx : k + (ny - 1) * nx;
+    n[3] = j < ny - 1 ? k + nx : k - (ny - 1) * nx;
 }
+
+// A thread's two cells of a level, by colour: place (-1: none), row and column, neighbours, face
+// coefficients (0 at a wall), inverse diagonal, Dirichlet-wall coefficient, right-hand side.
+struct TailPair {
+    int k[2], i[2], j[2], n[2][4];
+    float c[2][4], d[2], w[2], r[2];
+};
 
 template <class M0>
 __device__ __forceinline__ void tail_case(const DevCase* __restrict__ dc, int max_cells, int max_small,
                                           unsigned char* smem_raw, TailLevel* lv, MGLevel* geo) {
     if (pot_done(dc)) return;
     const CaseParams& P = dc->P;
-    const int L0 = dc->tail, n_lev = dc->nlev - L0;
+    const int L0 = dc->tail, n_lev = dc->nlev - L0, t = threadIdx.x;
     // per level, cell by cell: mu, right-hand side, correction, coefficients of the right and
-    // upper faces (0 at a wall), inverse diagonal; p and A p of the conjugate gradients; the
-    // neighbour table: cells to the left, right, below, above, and i, j
+    // upper faces (0 at a wall) and of Dirichlet walls, inverse diagonal; the residual of one
+    // level at a time; p and A p of the conjugate gradients
     float* mu = reinterpret_cast<float*>(smem_raw);
-    float *r = mu + max_cells, *e = r + max_cells, *cx = e + max_cells, *cy = cx + max_cells, *di = cy + max_cells;
-    float *p = di + max_cells, *Ap = p + max_small;
-    unsigned short* tab = reinterpret_cast<unsigned short*>(Ap + max_small);   // [max_small][6]
-    if (threadIdx.x < n_lev) {
-        int off = 0, tb = 0;
-        for (int l = 0; l < (int)threadIdx.x; ++l) {
-            const int n = dc->lev[L0 + l].nx * dc->lev[L0 + l].ny;
-            off += n;
-            if (n <= kWarpCells) tb += n;
-        }
-        const MGLevel g = dc->lev[L0 + threadIdx.x];
-        geo[threadIdx.x] = g;
-        lv[threadIdx.x] = TailLevel{g.nx, g.ny, off, g.ragged,
-                                    g.nx * g.ny <= kWarpCells || (int)threadIdx.x == n_lev - 1 ? tb : -1};
+    float *r = mu + max_cells, *e = r + max_cells, *cx = e + max_cells, *cy = cx + max_cells, *wl = cy + max_cells;
+    float *di = wl + max_cells, *res = di + max_cells, *p = res + max_cells, *Ap = p + max_small;
+    if (t < n_lev) {
+        int off = 0;
+        for (int l = 0; l < t; ++l) off += dc->lev[L0 + l].nx * dc->lev[L0 + l].ny;
+        const MGLevel g = dc->lev[L0 + t];
+        geo[t] = g;
+        lv[t] = TailLevel{g.nx, g.ny, off, g.ragged, max(32, ((g.nx * g.ny + 1) / 2 + 31) / 32 * 32)};
     }
     {
         const MGLevel& g = dc->lev[L0];
         if (sizeof(M0) == 8 && L0 == 0) {
             const double sc = dc->stats[ST_SCALE];
-            tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
+            tail_cells(g.nx, g.ny, [&](int i, int j, int k) {
                 const size_t q = (size_t)j * g.pitch + i;
                 mu[k] = (float)static_cast<const double*>(g.mu)[q];
                 r[k] = (float)(static_cast<const double*>(g.r)[q] * sc);
             });
         } else {
-            tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
+            tail_cells(g.nx, g.ny, [&](int i, int j, int k) {
                 const size_t q = (size_t)j * g.pitch + i;
                 mu[k] = static_cast<const float*>(g.mu)[q];
                 r[k] = static_cast<const float*>(g.r)[q];
@@ -934,7 +936,7 @@ __device__ __forceinline__ void tail_case(const DevCase* __restrict__ dc, int ma
     for (int l = 0; l + 1 < n_lev; ++l) {
         const TailLevel v = lv[l], c = lv[l + 1];
         const float* m = mu + v.off;
-        tail_cells(kTailNT, c.nx, c.ny, -1, [&](int I, int J, int K) {
+        tail_cells(c.nx, c.ny, [&](int I, int J, int K) {
             const int i0 = 2 * I, j0 = 2 * J, i1 = i0 + 1 < v.nx, j1 = j0 + 1 < v.ny;
             const float* q = m + j0 * v.nx + i0;
             float s = q[0];
@@ -944,244 +946,222 @@ __device__ __forceinline__ void tail_case(const DevCase* __restrict__ dc, int ma
         });
         __syncthreads();
     }
-    // coefficients of every level, and its neighbour table
+    // coefficients of every level
     for (int l = 0; l < n_lev; ++l) {
         const TailLevel v = lv[l];
         const MGLevel& g = geo[l];
         const float* m = mu + v.off;
-        tail_cells(kTailNT, v.nx, v.ny, -1, [&](int i, int j, int k) {
-            const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
-            const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
-            const int kn[4] = {kl, kr, kb, kt};
+        tail_cells(v.nx, v.ny, [&](int i, int j, int k) {
+            int n[4];
+            tail_neighbours(v.nx, v.ny, i, j, k, n);
             const bool in[4] = {per_x || i > 0, per_x || i < v.nx - 1, per_y || j > 0, per_y || j < v.ny - 1};
             const float mc = m[k];
-            float d = 0.f, c4[4];
+            float d = 0.f, wall = 0.f, c4[4];
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
                 c4[w] = 0.f;
                 if (in[w]) {
-                    c4[w] = 0.5f * (mc + m[kn[w]]);
+                    c4[w] = 0.5f * (mc + m[n[w]]);
                     if (v.ragged) c4[w] *= face_factor<float>(g, i, j, w, false);
                     d += c4[w];
                 } else if (dirichlet >> w & 1) {
-                    d += (v.ragged ? face_factor<float>(g, i, j, w, true) : 2.f) * mc;
+                    wall += (v.ragged ? face_factor<float>(g, i, j, w, true) : 2.f) * mc;
                 }
             }
             cx[v.off + k] = c4[1];
             cy[v.off + k] = c4[3];
-            di[v.off + k] = fdiv(1.f, d);
-            if (v.tab >= 0) {
-                unsigned short* t = tab + 6 * (v.tab + k);
-                t[0] = (unsigned short)kl;
-                t[1] = (unsigned short)kr;
-                t[2] = (unsigned short)kb;
-                t[3] = (unsigned short)kt;
-                t[4] = (unsigned short)i;
-                t[5] = (unsigned short)j;
-            }
+            wl[v.off + k] = wall;
+            di[v.off + k] = fdiv(1.f, d + wall);
         });
     }
     __syncthreads();
-    // sum_f c_f x_nb over a cell's faces (a wall face's coefficient is 0: the right face of the
-    // last column, the upper face of the last row)
-    auto nb_sum = [&](const TailLevel& v, const float* x, int k, int kl, int kr, int kb, int kt) {
+    auto meet = [&](int l) {   // the threads that own cells of level l
+        if (lv[l].nt == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(2 + l), "r"(lv[l].nt) : "memory");
+    };
+    TailPair q;
+    auto load = [&](int l) {
+        const TailLevel v = lv[l];
         const float *a = cx + v.off, *b = cy + v.off;
-        return (a[kl] * x[kl] + a[k] * x[kr]) + (b[kb] * x[kb] + b[k] * x[kt]);
-    };
-    // r - A x in differences, so that smooth x keeps its digits
-    auto residual = [&](const TailLevel& v, const MGLevel& g, const float* x, int i, int j, int k) {
-        const float *a = cx + v.off, *b = cy + v.off;
-        const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
-        const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
-        const float xc = x[k];
-        float ax = (a[kl] * (xc - x[kl]) + a[k] * (xc - x[kr])) + (b[kb] * (xc - x[kb]) + b[k] * (xc - x[kt]));
-        const bool at[4] = {!per_x && i == 0, !per_x && i == v.nx - 1, !per_y && j == 0, !per_y && j == v.ny - 1};
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-            if (at[w] && (dirichlet >> w & 1)) ax += (v.ragged ? face_factor<float>(g, i, j, w, true) : 2.f) * mu[v.off + k] * xc;
-        return r[v.off + k] - ax;
-    };
-    auto restrict_cell = [&](int l, int I, int J) {
-        const TailLevel v = lv[l];
-        float acc = 0.f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = 2 * I + (q & 1), j = 2 * J + (q >> 1);
-            if (i < v.nx && j < v.ny) acc += residual(v, geo[l], e + v.off, i, j, j * v.nx + i);
-        }
-        return acc;
-    };
-    auto prolong_cell = [&](int l, int i, int j) {
-        const TailLevel v = lv[l], c = lv[l + 1];
-        const float* xc = e + c.off;
-        const int I = i >> 1, J = j >> 1;
-        int di_ = (i & 1) ? 1 : -1, dj_ = (j & 1) ? 1 : -1;
-        float wx = 0.25f, wy = 0.25f;
-        if (v.ragged || c.ragged) {
-            prolong_axis<float>(i, v.nx, geo[l].wlx, c.nx, geo[l + 1].wlx, di_, wx);
-            prolong_axis<float>(j, v.ny, geo[l].wly, c.ny, geo[l + 1].wly, dj_, wy);
-        }
-        return ((1.f - wx) * (1.f - wy)) * xc[J * c.nx + I] +
-               (wx * (1.f - wy)) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J) +
-               ((1.f - wx) * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I, J + dj_) +
-               (wx * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J + dj_);
-    };
-    auto sweep = [&](int nt, int l, int colour) {
-        const TailLevel v = lv[l];
-        float* x = e + v.off;
-        tail_cells(nt, v.nx, v.ny, colour, [&](int i, int j, int k) {
-            const int kl = i > 0 ? k - 1 : k + v.nx - 1, kr = i < v.nx - 1 ? k + 1 : k - v.nx + 1;
-            const int kb = j > 0 ? k - v.nx : k + (v.ny - 1) * v.nx, kt = j < v.ny - 1 ? k + v.nx : k - (v.ny - 1) * v.nx;
-            x[k] = (r[v.off + k] + nb_sum(v, x, k, kl, kr, kb, kt)) * di[v.off + k];
-        });
-        tail_sync(nt);
-    };
-    const int lane = threadIdx.x & 31;
-    auto warp_sweep = [&](int l, int colour) {   // one warp
-        const TailLevel v = lv[l];
-        float* x = e + v.off;
         const int n = v.nx * v.ny;
-        for (int k = lane; k < n; k += 32) {
-            const unsigned short* t = tab + 6 * (v.tab + k);
-            if (((t[4] + t[5]) & 1) == colour) x[k] = (r[v.off + k] + nb_sum(v, x, k, t[0], t[1], t[2], t[3])) * di[v.off + k];
+        // colour of cell 2t: (i + j) & 1, which is k & 1 on rows of odd length
+        const int j0 = 2 * t / v.nx, c0 = v.nx & 1 ? 0 : j0 & 1;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int k = 2 * t + (s ^ c0);
+            q.k[s] = k < n ? k : -1;
+            if (k >= n) continue;
+            const int j = k / v.nx, i = k - j * v.nx;
+            q.i[s] = i;
+            q.j[s] = j;
+            tail_neighbours(v.nx, v.ny, i, j, k, q.n[s]);
+            q.c[s][0] = a[q.n[s][0]];
+            q.c[s][1] = a[k];
+            q.c[s][2] = b[q.n[s][2]];
+            q.c[s][3] = b[k];
+            q.d[s] = di[v.off + k];
+            q.w[s] = wl[v.off + k];
+            q.r[s] = r[v.off + k];
         }
-        __syncwarp();
     };
-    int small = 0, twice = 0;   // first level of one warp, first level of the part that runs twice
-    while (small < n_lev - 1 && lv[small].tab < 0) ++small;
-    while (twice < n_lev - 1 && lv[twice].nx * lv[twice].ny > kPassCells) ++twice;
-    auto down = [&](int nt, int l, bool fresh) {
-        const TailLevel v = lv[l], c = lv[l + 1];
-        float* x = e + v.off;
-        if (fresh) {   // first sweep from zero: the first colour's neighbours are zero
-            tail_cells(nt, v.nx, v.ny, -1, [&](int i, int j, int k) { x[k] = ((i + j) & 1) ? 0.f : r[v.off + k] * di[v.off + k]; });
-            tail_sync(nt);
+    auto relaxed = [&](int s, const float* x) {   // the sweep's new value of the cell of colour s
+        return (q.r[s] + ((q.c[s][0] * x[q.n[s][0]] + q.c[s][1] * x[q.n[s][1]]) +
+                          (q.c[s][2] * x[q.n[s][2]] + q.c[s][3] * x[q.n[s][3]]))) * q.d[s];
+    };
+    auto half = [&](int l, int s, float* x) {
+        if (q.k[s] >= 0) x[q.k[s]] = relaxed(s, x);
+        meet(l);
+    };
+    auto restrict_to = [&](int l, int k) {   // cell k of level l: the residual of its children on level l - 1
+        const TailLevel v = lv[l - 1], c = lv[l];
+        const int J = k / c.nx, I = k - J * c.nx, i1 = 2 * I + 1 < v.nx, j1 = 2 * J + 1 < v.ny;
+        const float* y = res + 2 * J * v.nx + 2 * I;
+        float s = y[0];
+        if (i1) s += y[1];
+        if (j1) s += i1 ? y[v.nx] + y[v.nx + 1] : y[v.nx];
+        r[c.off + k] = s;
+    };
+    auto down = [&](int l, bool fresh) {
+        load(l);
+        float* x = e + lv[l].off;
+        if (fresh) {   // from zero: the first colour's neighbours are zero
+            if (q.k[0] >= 0) x[q.k[0]] = q.r[0] * q.d[0];
+            if (q.k[1] >= 0) x[q.k[1]] = 0.f;   // (read with a zero coefficient across a wall)
+            meet(l);
         } else {
-            sweep(nt, l, 0);
+            half(l, 0, x);
         }
-        sweep(nt, l, 1);
-        for (int s = 1; s < kFNu; ++s) {
-            sweep(nt, l, 0);
-            sweep(nt, l, 1);
+        half(l, 1, x);
+#pragma unroll
+        for (int n = 1; n < kFNu; ++n) {
+            half(l, 0, x);
+            half(l, 1, x);
         }
-        tail_cells(nt, c.nx, c.ny, -1, [&](int I, int J, int K) { r[c.off + K] = restrict_cell(l, I, J); });
-        tail_sync(nt);
+#pragma unroll
+        for (int s = 0; s < 2; ++s)   // r - A x in differences, so that smooth x keeps its digits
+            if (q.k[s] >= 0) {
+                const float xc = x[q.k[s]];
+                res[q.k[s]] = q.r[s] - (((q.c[s][0] * (xc - x[q.n[s][0]]) + q.c[s][1] * (xc - x[q.n[s][1]])) +
+                                         (q.c[s][2] * (xc - x[q.n[s][2]]) + q.c[s][3] * (xc - x[q.n[s][3]]))) + q.w[s] * xc);
+            }
+        meet(l);
+        const TailLevel c = lv[l + 1];
+        const int n = c.nx * c.ny;
+        if (l + 1 < n_lev - 1) {   // each owner its own cells, which it loads next
+            if (2 * t < n) restrict_to(l + 1, 2 * t);
+            if (2 * t + 1 < n) restrict_to(l + 1, 2 * t + 1);
+        } else if (t < 32) {
+            for (int k = t; k < n; k += 32) restrict_to(l + 1, k);
+        }
     };
-    auto up = [&](int nt, int l) {
-        const TailLevel v = lv[l];
+    auto up = [&](int l) {
+        meet(l);   // the coarser level is done
+        load(l);
+        const TailLevel v = lv[l], c = lv[l + 1];
         float* x = e + v.off;
-        tail_cells(nt, v.nx, v.ny, -1, [&](int i, int j, int k) { x[k] += prolong_cell(l, i, j); });
-        tail_sync(nt);
-        for (int s = 0; s < kFNu; ++s) {
-            sweep(nt, l, 0);
-            sweep(nt, l, 1);
+        const float* xc = e + c.off;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            if (q.k[s] < 0) continue;
+            const int i = q.i[s], j = q.j[s], I = i >> 1, J = j >> 1;
+            int di_ = (i & 1) ? 1 : -1, dj_ = (j & 1) ? 1 : -1;
+            float wx = 0.25f, wy = 0.25f;
+            if (v.ragged || c.ragged) {
+                prolong_axis<float>(i, v.nx, geo[l].wlx, c.nx, geo[l + 1].wlx, di_, wx);
+                prolong_axis<float>(j, v.ny, geo[l].wly, c.ny, geo[l + 1].wly, dj_, wy);
+            }
+            x[q.k[s]] += ((1.f - wx) * (1.f - wy)) * xc[J * c.nx + I] +
+                         (wx * (1.f - wy)) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J) +
+                         ((1.f - wx) * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I, J + dj_) +
+                         (wx * wy) * coarse_at<float>(walls, xc, c.nx, c.ny, c.nx, I + di_, J + dj_);
+        }
+        meet(l);
+#pragma unroll
+        for (int n = 0; n < kFNu; ++n) {
+            half(l, 0, x);
+            half(l, 1, x);
         }
     };
-    auto one_warp = [&](bool fresh_top) {   // levels small to the coarsest and back
-        for (int l = small; l + 1 < n_lev; ++l) {
-            const TailLevel v = lv[l], c = lv[l + 1];
-            float* x = e + v.off;
-            const int n = v.nx * v.ny, nc = c.nx * c.ny;
-            if (fresh_top || l > small) {
-                for (int k = lane; k < n; k += 32) {
-                    const unsigned short* t = tab + 6 * (v.tab + k);
-                    x[k] = ((t[4] + t[5]) & 1) ? 0.f : r[v.off + k] * di[v.off + k];
-                }
-                __syncwarp();
-            } else {
-                warp_sweep(l, 0);
-            }
-            warp_sweep(l, 1);
-            for (int s = 1; s < kFNu; ++s) {
-                warp_sweep(l, 0);
-                warp_sweep(l, 1);
-            }
-            for (int k = lane; k < nc; k += 32) {
-                const unsigned short* t = tab + 6 * (c.tab + k);
-                r[c.off + k] = restrict_cell(l, t[4], t[5]);
-            }
-            __syncwarp();
-        }
-        const TailLevel v = lv[n_lev - 1];
+    auto coarsest = [&] {   // one warp
+        const int l = n_lev - 1;
+        const TailLevel v = lv[l];
         const int n = v.nx * v.ny;
-        float *x = e + v.off, *q = r + v.off;
+        float *x = e + v.off, *b = r + v.off;
+        __syncwarp();
+        for (int k = t; k < n; k += 32) x[k] = 0.f;
+        __syncwarp();
         if (n <= kTinyCells) {
-            for (int k = lane; k < n; k += 32) x[k] = 0.f;
-            __syncwarp();
-            for (int s = 0; s < 2 * kFNu; ++s) {
-                warp_sweep(n_lev - 1, 0);
-                warp_sweep(n_lev - 1, 1);
-            }
-        } else {   // conjugate gradients
-            const float* dg = di + v.off;
-            float rr = 0.f;
-            for (int k = lane; k < n; k += 32) {
-                p[k] = q[k];
-                x[k] = 0.f;
-                rr += q[k] * q[k];
-            }
-            rr = warp_allsum(rr);
-            __syncwarp();
-            const float rr0 = rr;
-            const float tol2 = 1e-6f;   // a coarse correction needs only a few digits (as the block version)
-            const int maxit = 4 * (v.nx + v.ny) + 100;
-            for (int it = 0; it < maxit && rr > tol2 * rr0 && rr > 0.f; ++it) {
-                float pAp = 0.f;
-                for (int k = lane; k < n; k += 32) {
-                    const unsigned short* t = tab + 6 * (v.tab + k);
-                    const float y = fdiv(p[k], dg[k]) - nb_sum(v, p, k, t[0], t[1], t[2], t[3]);
-                    Ap[k] = y;
-                    pAp += p[k] * y;
-                }
-                pAp = warp_allsum(pAp);
-                const float alpha = rr / pAp;
-                float rn = 0.f;
-                for (int k = lane; k < n; k += 32) {
-                    x[k] += alpha * p[k];
-                    const float rk = q[k] - alpha * Ap[k];
-                    q[k] = rk;
-                    rn += rk * rk;
-                }
-                rn = warp_allsum(rn);
-                const float beta = rn / rr;
-                rr = rn;
-                __syncwarp();   // every lane's reads of p for A p are done
-                for (int k = lane; k < n; k += 32) p[k] = q[k] + beta * p[k];
+            load(l);
+            for (int h = 0; h < 4 * kFNu; ++h) {
+                const int s = h & 1;
+                const float y = q.k[s] >= 0 ? relaxed(s, x) : 0.f;
+                __syncwarp();   // (a periodic axis of odd length joins cells of one colour)
+                if (q.k[s] >= 0) x[q.k[s]] = y;
                 __syncwarp();
             }
+            return;
         }
-        for (int l = n_lev - 2; l >= small; --l) {
-            const TailLevel w = lv[l];
-            float* y = e + w.off;
-            for (int k = lane; k < w.nx * w.ny; k += 32) {
-                const unsigned short* t = tab + 6 * (w.tab + k);
-                y[k] += prolong_cell(l, t[4], t[5]);
+        // conjugate gradients
+        const float *a = cx + v.off, *c = cy + v.off, *dg = di + v.off;
+        float rr = 0.f;
+        for (int k = t; k < n; k += 32) {
+            p[k] = b[k];
+            rr += b[k] * b[k];
+        }
+        rr = warp_allsum(rr);
+        __syncwarp();
+        const float rr0 = rr;
+        const float tol2 = 1e-6f;   // a coarse correction needs only a few digits (as the block version)
+        const int maxit = 4 * (v.nx + v.ny) + 100;
+        for (int it = 0; it < maxit && rr > tol2 * rr0 && rr > 0.f; ++it) {
+            float pAp = 0.f;
+            for (int k = t; k < n; k += 32) {
+                const int j = k / v.nx, i = k - j * v.nx;
+                int m[4];
+                tail_neighbours(v.nx, v.ny, i, j, k, m);
+                const float y = fdiv(p[k], dg[k]) - ((a[m[0]] * p[m[0]] + a[k] * p[m[1]]) + (c[m[2]] * p[m[2]] + c[k] * p[m[3]]));
+                Ap[k] = y;
+                pAp += p[k] * y;
             }
+            pAp = warp_allsum(pAp);
+            const float alpha = rr / pAp;
+            float rn = 0.f;
+            for (int k = t; k < n; k += 32) {
+                x[k] += alpha * p[k];
+                const float rk = b[k] - alpha * Ap[k];
+                b[k] = rk;
+                rn += rk * rk;
+            }
+            rn = warp_allsum(rn);
+            const float beta = rn / rr;
+            rr = rn;
+            __syncwarp();   // every lane's reads of p for A p are done
+            for (int k = t; k < n; k += 32) p[k] = b[k] + beta * p[k];
             __syncwarp();
-            for (int s = 0; s < kFNu; ++s) {
-                warp_sweep(l, 0);
-                warp_sweep(l, 1);
-            }
         }
     };
-    const int top = min(twice, small);
-    for (int l = 0; l < top; ++l) down(kTailNT, l, true);
-    if (threadIdx.x < kTailFew) {   // levels of at most kPassCells cells: the first warps
+    // levels [0, mine) are the ones this thread owns cells of; from level `twice` the part that
+    // runs twice
+    int twice = 0, mine = 0;
+    while (twice < n_lev - 1 && lv[twice].nx * lv[twice].ny > kPassCells) ++twice;
+    while (mine < n_lev - 1 && t < lv[mine].nt) ++mine;
+    const int top = min(twice, mine);
+    for (int l = 0; l < top; ++l) down(l, true);
+    if (twice < n_lev - 1 ? mine > twice : t < 32) {
         const int passes = twice < n_lev - 1 ? kTailPasses : 1;
         for (int pass = 0; pass < passes; ++pass) {
-            for (int l = twice; l < small; ++l) down(kTailFew, l, pass == 0 || l > twice);
-            if (threadIdx.x < 32) one_warp(pass == 0 || small > twice);
-            tail_sync(kTailFew);
-            for (int l = small - 1; l >= twice; --l) up(kTailFew, l);
+            for (int l = twice; l < mine; ++l) down(l, pass == 0 || l > twice);
+            if (t < 32) coarsest();
+            for (int l = mine - 1; l >= twice; --l) up(l);
         }
     }
+    for (int l = top - 1; l >= 0; --l) up(l);
     __syncthreads();
-    for (int l = top - 1; l >= 0; --l) up(kTailNT, l);
     const MGLevel& g = geo[0];
-    tail_cells(kTailNT, g.nx, g.ny, -1, [&](int i, int j, int k) {
-        const unsigned q = (unsigned)j * (unsigned)g.pitch + (unsigned)i;
-        if (L0 == 0) add_correction<M0>(dc, q, e[k]);
-        else static_cast<float*>(g.e)[q] = e[k];
+    tail_cells(g.nx, g.ny, [&](int i, int j, int k) {
+        const unsigned o = (unsigned)j * (unsigned)g.pitch + (unsigned)i;
+        if (L0 == 0) add_correction<M0>(dc, o, e[k]);
+        else static_cast<float*>(g.e)[o] = e[k];
     });
 }
 
@@ -1477,7 +1457,7 @@ cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, 
 }
 
 static size_t tail_bytes(int max_cells, int max_small) {
-    return (size_t)6 * max_cells * sizeof(float) + (size_t)max_small * (2 * sizeof(float) + 6 * sizeof(short));
+    return ((size_t)8 * max_cells + (size_t)2 * max_small) * sizeof(float);
 }
 
 cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* ids, int ncases, int max_cells, int max_small,
