@@ -550,8 +550,8 @@ def main(argv=None):
                     help="skip the multigrid versus pseudo-time magnetic LBFS comparison")
     ap.add_argument("--tile", type=int, default=-1, help="stage tile shape id; -1: autotune")
     ap.add_argument("--plain-cycles", action="store_true",
-                    help="warm potential cycles as plain launches (for kernel profilers, which cannot follow "
-                         "conditional graph nodes)")
+                    help="warm potential cycles as plain launches (so that a kernel profiler shows each "
+                         "phase of a cycle)")
     ap.add_argument("--graph", type=int, default=0,
                     help="1: replay recorded CUDA graphs (disables the per-kernel timing)")
     args = ap.parse_args(argv)

@@ -1,7 +1,7 @@
 // lbfs_api.cu -- host implementation of the C ABI declared in include/lbfs.h:
-// context and case management, device memory layout, tile work lists for batched
-// cases, and the per-step schedule (potential refinement, three Runge-Kutta stages,
-// step-end statistics), optionally recorded once as a CUDA graph and replayed.
+// context and case management, device memory layout, lists of strips and tiles for batched
+// cases, and the per-step schedule (potential refinement, three Runge-Kutta stages, the last
+// with the step's statistics), optionally recorded once as a CUDA graph and replayed.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -75,9 +75,8 @@ struct lbfs_ctx {
     bool pot_fresh = true; // a state was set since the last full potential solve
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
-    int64_t graph_launches = 0;       // kernel nodes in one recorded step, the cycle body's aside
+    int64_t graph_launches = 0;       // kernel nodes in one recorded step
     cudaStream_t cap_stream = nullptr; // private stream used to record the graph
-    bool capturing = false;           // launches are being recorded into a graph
     // kernel timing (events on the context stream)
     bool timing = false;
     double t_ms[3] = {0, 0, 0};
@@ -591,12 +590,10 @@ lbfs_status record_graph(lbfs_ctx* ctx) {
     cudaStream_t user = ctx->stream;
     const int64_t l0 = ctx->launches;
     ctx->stream = ctx->cap_stream;
-    ctx->capturing = true;
     cudaError_t e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal);
     lbfs_status r = e == cudaSuccess ? one_step(ctx) : LBFS_ECUDA;
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &g);
-    ctx->capturing = false;
     ctx->stream = user;
     ctx->graph_launches = ctx->launches - l0;
     ctx->launches = l0;
@@ -757,7 +754,7 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     }
     if (ctx->prec == 0) {
         add((void**)&hd.phi64, cells * sizeof(double));
-        add((void**)&hd.phi_prev64, cells * sizeof(double));
+        add((void**)&hd.phi_prev64, 2 * cells * sizeof(double));
     } else {
         add(&hd.phi, cells * rs);
         add((void**)&hd.phi_lo, cells * sizeof(float));

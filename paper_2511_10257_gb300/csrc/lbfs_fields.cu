@@ -1,6 +1,6 @@
 // lbfs_fields.cu -- per-case utility kernels: initial condition, field export and
-// import in FP64, the potential coefficient of a state, and the step-end statistics
-// (Eq. 51 liquid fraction of the droplet, sums of C and H_e, freezing time).
+// import in FP64, the potential coefficient of a state, its statistics (Eq. 51 liquid
+// fraction of the droplet, sums of C and H_e) and the Sec. 5 diagnostics.
 #include "lbfs_kernels.h"
 
 namespace lbfs {

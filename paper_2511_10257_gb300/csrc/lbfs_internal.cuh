@@ -8,8 +8,8 @@
 namespace lbfs {
 
 constexpr int kMaxLevels = 16;
-constexpr int kRedN = 6;        // per-tile partial sums of the step-end reduction
-constexpr int kFinChunks = 32;  // blocks per case that reduce the tile partials
+constexpr int kRedN = 6;        // partial sums of a strip in the step-end reduction
+constexpr int kFinChunks = 32;  // blocks per case that sum a stored state's statistics
 constexpr int kStatN = 20;      // per-case device statistics slots
 
 // statistics slots (FP64, per case).  ST_POT_RESID_MAX, ST_POT_CYCLES_SUM and
