@@ -498,7 +498,8 @@ __device__ __forceinline__ void add_correction(const DevCase* dc, unsigned k, fl
 // each, so after kFNu full sweeps the tile (plus one cell) holds exactly the values the
 // sweeps over the whole level would give.  Down leg: pre-smooth from e = 0, store e,
 // restrict r - A e to the next level.  Up leg: add the bilinear prolongation of the
-// coarse correction, post-smooth, store e.
+// coarse correction, post-smooth, store eu (neighbouring tiles still read e) or, on the fine level,
+// add to phi.
 constexpr int kFNu = 2;
 constexpr int kHD = 2 * kFNu + 1, kHU = 2 * kFNu;
 
@@ -1181,7 +1182,8 @@ __global__ void __launch_bounds__(kTailNT) k_tail(const DevCase* __restrict__ ca
 // dependent phases: a leg's tile takes kLegNT threads, a coarse solve a block, a residual strip
 // a warp.  When the check before it found every case converged the kernel returns at once.
 // The phases run the same code on the same data as the kernels of their own: the potential is
-// the same bit for bit.
+// the same bit for bit.  Bound by latency: a cycle on 128 x 64 takes 57 us, against 46 as kernels of a
+// recorded graph, but a step that needs none pays 5 us where a conditional graph node took 16.
 constexpr int kLegNT = 256, kLegGroups = kTailNT / kLegNT;
 
 // All blocks of the grid arrive (sync[0] counts them; it starts a launch at zero and only
