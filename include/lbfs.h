@@ -57,7 +57,9 @@ typedef struct lbfs_config {
     int32_t use_graph;       /* 1: record the step as a CUDA graph and replay it           */
     void*   cuda_stream;     /* borrowed cudaStream_t; NULL: the context creates its own   */
     void* (*dev_alloc)(size_t bytes, void* user);  /* optional device allocator, e.g. a   */
-    void  (*dev_free)(void* ptr, void* user);      /* framework's caching allocator       */
+    void  (*dev_free)(void* ptr, void* user);      /* framework's caching allocator; the
+                                memory is used on cuda_stream at once, so no other stream
+                                may have work left on it                                   */
     void*   alloc_user;
     int32_t mg_max_cycles;   /* refinement cycles of a potential solve after a state is set,
                                 checked on the device (0: 40)                              */

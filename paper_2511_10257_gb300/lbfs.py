@@ -146,7 +146,8 @@ class Solver:
 
     stream: an int cudaStream_t handle to borrow (e.g. torch's current stream), or
     None for a stream owned by the context.  torch_alloc: route device memory
-    through torch's caching allocator.
+    through torch's caching allocator (each allocation, at set-up, waits for torch's
+    current stream).
     """
 
     def __init__(self, precision: int = FP64, max_cases: int = 1, device: int = 0,
@@ -171,7 +172,11 @@ class Solver:
             import torch
 
             def _alloc(nbytes, user):
-                return torch.cuda.caching_allocator_alloc(int(nbytes), device)
+                ptr = torch.cuda.caching_allocator_alloc(int(nbytes), device)
+                # the block is ordered on torch's current stream, on which kernels may still use
+                # the tensor that held it before; the library uses it on its own stream at once
+                torch.cuda.current_stream(device).synchronize()
+                return ptr
 
             def _free(ptr, user):
                 torch.cuda.caching_allocator_delete(ptr)

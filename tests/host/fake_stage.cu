@@ -1,0 +1,32 @@
+// fake_stage.cu -- the stage kernel's launches in the tests of the host code (fake_cuda.cpp): a
+// line in the log, which for a batch compares the strips that each case's table counts with those
+// in the list.
+#include <map>
+#include <string>
+
+#include "lbfs_kernels.h"
+#include "lbfs_stage.cuh"
+
+extern "C" void fake_say(const char* what, cudaStream_t s, const char* more);
+
+namespace lbfs {
+
+template <class R, bool HALF, bool UNI>
+cudaError_t stage_launch(const StageCase<R>&, const StageCase<R>* cases, const TileRef* tiles, int ntiles, int, int,
+                         cudaStream_t st) {
+    std::map<int, int> n;
+    for (int t = 0; t < ntiles; ++t) ++n[tiles[t].case_id];
+    std::string more = UNI ? "one" : "batch";
+    for (const auto& c : n)
+        if (!UNI && cases[c.first].strips != c.second)
+            more += " case " + std::to_string(c.first) + ": " + std::to_string(cases[c.first].strips) + " strips of " +
+                    std::to_string(c.second);
+    fake_say("stage", st, more.c_str());
+    return cudaSuccess;
+}
+#define FAKE_STAGE(R, H, U) \
+    template cudaError_t stage_launch<R, H, U>(const StageCase<R>&, const StageCase<R>*, const TileRef*, int, int, int, cudaStream_t);
+FAKE_STAGE(float, true, true) FAKE_STAGE(float, false, true) FAKE_STAGE(float, true, false) FAKE_STAGE(float, false, false)
+FAKE_STAGE(double, true, true) FAKE_STAGE(double, false, true) FAKE_STAGE(double, true, false) FAKE_STAGE(double, false, false)
+
+}  // namespace lbfs

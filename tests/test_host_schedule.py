@@ -1,0 +1,55 @@
+"""The host code of the library followed call by call on a fake CUDA runtime (tests/hostlib.py):
+what orders its memory, what its kernels are launched with, and what it does when a call fails."""
+import ctypes as ct
+
+import pytest
+
+import hostlib
+from paper_2511_10257_gb300 import inputs as I
+from paper_2511_10257_gb300 import lbfs
+
+BOTH = [lbfs.FP64, lbfs.MIXED]
+
+
+@pytest.fixture(scope="module")
+def host_lib(tmp_path_factory):
+    return hostlib.build(tmp_path_factory.mktemp("host"))
+
+
+@pytest.fixture
+def fake(host_lib, monkeypatch):
+    monkeypatch.setattr(lbfs, "_lib", None)
+    f = hostlib.Fake(lbfs.load(host_lib))
+    f.clear()
+    return f
+
+
+def _case(nx=64, ny=32, **kw):
+    return I.case(nx, ny, radius=9.0, H0=0.03, field_angle_deg=40.0, **kw)
+
+
+def test_torch_memory_is_free_of_pending_work_before_it_is_used(fake, monkeypatch):
+    """A block of torch's caching allocator may still be in use by kernels queued on torch's
+    current stream; the library's stream is not ordered behind them."""
+    torch = pytest.importorskip("torch")
+    libc = ct.CDLL(None)
+    libc.malloc.restype, libc.malloc.argtypes, libc.free.argtypes = ct.c_void_p, [ct.c_size_t], [ct.c_void_p]
+    calls = []
+
+    class Stream:
+        def synchronize(self):
+            calls.append("waited")
+
+    def alloc(n, device):
+        calls.append("allocated")
+        return libc.malloc(n)
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", alloc)
+    monkeypatch.setattr(torch.cuda, "caching_allocator_delete", libc.free)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: Stream())
+    s = lbfs.Solver(precision=lbfs.MIXED, max_cases=1, torch_alloc=True)
+    s.set_case(0, _case())
+    s.step(1)
+    s.fields(0, [I.C])
+    s.close()
+    assert len(calls) > 6 and calls == ["allocated", "waited"] * (len(calls) // 2)
