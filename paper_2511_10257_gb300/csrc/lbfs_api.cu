@@ -305,16 +305,29 @@ void fill_stage(const DevCase& d, StageCase<R>& c) {
     }
 }
 
-// Upload the concatenated tile lists of all defined cases.
-lbfs_status rebuild(lbfs_ctx* ctx) {
-    drop_graph(ctx);
-    std::vector<TileRef> st;
+// The lists of strips, tiles and cases that the kernels read, on the host.
+struct Lists {
+    std::vector<TileRef> stage, resid, mg;
+    std::vector<int> tails, others;
+    std::vector<std::vector<TileRef>> legs;   // fused V-cycle tiles per level
+};
+
+// Make the concatenated lists of all defined cases and send them, with the counts in the cases'
+// tables that depend on them, in the order of the stream whose kernels read them (a copy on the
+// default stream may return before its data has arrived, and a non-blocking stream does not wait
+// for it).
+lbfs_status make_lists(lbfs_ctx* ctx, Lists& lists) {
+    auto send = [&](void* dst, const void* src, size_t bytes) {
+        return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream) == cudaSuccess;
+    };
+    std::vector<TileRef>& st = lists.stage;
     long long row_warps = 0;   // strips of one row's height over all cases
     for (const Slot& s : ctx->slots)
         if (s.defined) row_warps += (long long)((s.hd.P.nx + kStripW - 1) / kStripW) * s.hd.P.ny;
     const int TX = kStripW, TY = stage_rows(ctx->prec, ctx->tile, row_warps, ctx->sm_count);
     ctx->rows = TY;
-    std::vector<int> pot, tails, others;
+    std::vector<int> pot;
+    std::vector<int>&tails = lists.tails, &others = lists.others;
     int active = 0, depth = 0, tail_cells = 0, tail_small = 0, coarsest = 0;
     int half = 1;
     // The residual's strips: 64 rows, or fewer while all of them run at once (24 warps an SM)
@@ -324,7 +337,7 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             res_warps += (long long)((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * s.hd.P.ny;
     int res_rows = kResidMinRows;
     while (res_rows < 64 && res_warps > 24LL * ctx->sm_count * res_rows) res_rows *= 2;
-    std::vector<TileRef> rt;
+    std::vector<TileRef>& rt = lists.resid;
     for (int c = 0; c < (int)ctx->slots.size(); ++c) {
         Slot& s = ctx->slots[c];
         if (!s.defined) continue;
@@ -333,13 +346,13 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
             s.sf.strips = s.sd.strips = strips;
             const void* sc = ctx->prec == 0 ? (const void*)&s.sd : (const void*)&s.sf;
             const size_t scb = ctx->prec == 0 ? sizeof(s.sd) : sizeof(s.sf);
-            if (cudaMemcpy(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb, cudaMemcpyHostToDevice) != cudaSuccess)
+            if (!send(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb))
                 return fail(ctx, LBFS_ECUDA, "case table update failed");
         }
         const int res = ((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * ((s.hd.P.ny + res_rows - 1) / res_rows);
         if (res != s.hd.mg_strips) {
             s.hd.mg_strips = res;
-            if (cudaMemcpy(ctx->d_cases + c, &s.hd, sizeof(DevCase), cudaMemcpyHostToDevice) != cudaSuccess)
+            if (!send(ctx->d_cases + c, &s.hd, sizeof(DevCase)))
                 return fail(ctx, LBFS_ECUDA, "case table update failed");
         }
         ++active;
@@ -366,8 +379,9 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
                 for (int x = 0; x < s.hd.P.nx; x += kResidStripW) rt.push_back(TileRef{c, x, y, slot++});
         }
     }
-    std::vector<TileRef> mg;
-    std::vector<std::vector<TileRef>> ft(depth);
+    std::vector<TileRef>& mg = lists.mg;
+    std::vector<std::vector<TileRef>>& ft = lists.legs;
+    ft.resize(depth);
     if (ctx->prec == 0)
         for (int c : pot) {
             const CaseParams& P = ctx->slots[c].hd.P;
@@ -406,7 +420,7 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
         if (bytes == 0) return true;
         *dst = dalloc(ctx, bytes);
         if (!*dst) return false;
-        return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+        return send(*dst, src, bytes);
     };
     if (!upload((void**)&ctx->d_stage_tiles, st.data(), st.size() * sizeof(TileRef)) ||
         !upload((void**)&ctx->d_mg_tiles, mg.data(), mg.size() * sizeof(TileRef)) ||
@@ -435,6 +449,16 @@ lbfs_status rebuild(lbfs_ctx* ctx) {
     ctx->max_depth = depth;
     ctx->coarsest_cells = coarsest;
     ctx->half = half;
+    return LBFS_OK;
+}
+
+lbfs_status rebuild(lbfs_ctx* ctx) {
+    drop_graph(ctx);
+    Lists lists;
+    const lbfs_status r = make_lists(ctx, lists);
+    const cudaError_t e = cudaStreamSynchronize(ctx->stream);   // `lists` outlives its copies
+    if (r != LBFS_OK) return r;
+    if (e != cudaSuccess) return fail(ctx, LBFS_ECUDA, std::string("tile list upload: ") + cudaGetErrorString(e));
     ctx->dirty = false;
     return LBFS_OK;
 }

@@ -53,3 +53,24 @@ def test_torch_memory_is_free_of_pending_work_before_it_is_used(fake, monkeypatc
     s.fields(0, [I.C])
     s.close()
     assert len(calls) > 6 and calls == ["allocated", "waited"] * (len(calls) // 2)
+
+
+@pytest.mark.parametrize("precision", BOTH)
+@pytest.mark.parametrize("graph", [False, True])
+def test_lists_arrive_before_the_kernels_that_read_them(fake, precision, graph):
+    """Every upload is in the order of the kernels' own stream (one on the default stream is not
+    ordered before a non-blocking stream's kernels) and has ended before its host copy goes."""
+    s = lbfs.Solver(precision=precision, max_cases=2, use_graph=graph)
+    for k in range(2):
+        s.set_case(k, _case(300, 150))
+    fake.clear()
+    s.step(2)
+    s.autotune(1)
+    s.close()
+    log = fake.log()
+    assert not [w for w in log if w[0] == "copy-unordered"]
+    stream = {w[1] for w in log if w[0] == "launch"} - {w[1] for w in log if w[0] == "record"}
+    assert len(stream) == 1 and {w[1] for w in log if w[0] == "copy"} == stream
+    kinds = [w[0] for w in log]
+    uploads = [k for k in range(kinds.index("set")) if kinds[k] == "copy"]
+    assert uploads and "sync" in kinds[uploads[-1]:kinds.index("set")]
