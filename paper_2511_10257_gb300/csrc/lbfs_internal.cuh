@@ -312,15 +312,19 @@ __device__ __forceinline__ DSum<R> block_sum0(DSum<R> v, typename DSum<R>::Slot*
     return tot;
 }
 
-// whether this warp is the last of n to arrive at the ticket, which it then clears
+// Whether this warp is the last of n to arrive at the ticket, which it then clears.  The warp's
+// barriers extend what lane 0's fences order to all its lanes (a shuffle alone orders no memory):
+// what any lane wrote before is visible to the last warp, all of whose lanes may read it after.
 __device__ __forceinline__ bool last_of(unsigned* ticket, int n, int lane) {
     unsigned last = 0;
+    __syncwarp();
     if (lane == 0) {
         __threadfence();
         last = atomicAdd(ticket, 1u) == (unsigned)(n - 1);
         if (last) *ticket = 0u;
         __threadfence();
     }
+    __syncwarp();
     return __shfl_sync(0xffffffffu, last, 0) != 0;
 }
 
