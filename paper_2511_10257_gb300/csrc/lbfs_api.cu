@@ -341,20 +341,15 @@ lbfs_status make_lists(lbfs_ctx* ctx, Lists& lists) {
     for (int c = 0; c < (int)ctx->slots.size(); ++c) {
         Slot& s = ctx->slots[c];
         if (!s.defined) continue;
-        const int strips = ((s.hd.P.nx + TX - 1) / TX) * ((s.hd.P.ny + TY - 1) / TY);
-        if (strips != s.sf.strips) {
-            s.sf.strips = s.sd.strips = strips;
-            const void* sc = ctx->prec == 0 ? (const void*)&s.sd : (const void*)&s.sf;
-            const size_t scb = ctx->prec == 0 ? sizeof(s.sd) : sizeof(s.sf);
-            if (!send(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb))
-                return fail(ctx, LBFS_ECUDA, "case table update failed");
-        }
-        const int res = ((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * ((s.hd.P.ny + res_rows - 1) / res_rows);
-        if (res != s.hd.mg_strips) {
-            s.hd.mg_strips = res;
-            if (!send(ctx->d_cases + c, &s.hd, sizeof(DevCase)))
-                return fail(ctx, LBFS_ECUDA, "case table update failed");
-        }
+        // the counts of the kernels' last-arriver sums, on the device after every rebuild, whatever
+        // the tables held (lbfs_set_case clears them)
+        s.hd.mg_strips = ((s.hd.P.nx + kResidStripW - 1) / kResidStripW) * ((s.hd.P.ny + res_rows - 1) / res_rows);
+        s.sf.strips = s.sd.strips = ((s.hd.P.nx + TX - 1) / TX) * ((s.hd.P.ny + TY - 1) / TY);
+        const void* sc = ctx->prec == 0 ? (const void*)&s.sd : (const void*)&s.sf;
+        const size_t scb = ctx->prec == 0 ? sizeof(s.sd) : sizeof(s.sf);
+        if (!send(ctx->d_cases + c, &s.hd, sizeof(DevCase)) ||
+            !send(static_cast<char*>(ctx->d_stage_cases) + c * scb, sc, scb))
+            return fail(ctx, LBFS_ECUDA, "case table update failed");
         ++active;
         if (s.hd.P.dts != 0.5) half = 0;
         int slot = 0;

@@ -74,3 +74,39 @@ def test_lists_arrive_before_the_kernels_that_read_them(fake, precision, graph):
     kinds = [w[0] for w in log]
     uploads = [k for k in range(kinds.index("set")) if kinds[k] == "copy"]
     assert uploads and "sync" in kinds[uploads[-1]:kinds.index("set")]
+
+
+@pytest.mark.parametrize("precision", BOTH)
+@pytest.mark.parametrize("tune", [False, True])
+def test_a_redefined_case_keeps_its_strip_count(fake, precision, tune):
+    """A batch launch reads a case's strip count from its table, which defining the case clears."""
+    s = lbfs.Solver(precision=precision, max_cases=2)
+    for k in range(2):
+        s.set_case(k, _case())
+    if tune:
+        s.autotune(1)
+    else:
+        s.step(1)
+    s.set_case(0, _case(stefan=0.7))   # the same grid, so as many strips as before
+    fake.clear()
+    s.step(1)
+    s.close()
+    stages = [w for w in fake.log() if w[0] == "stage"]
+    assert len(stages) == 3 and all(w[2:] == ["batch"] for w in stages), stages
+
+
+def test_a_failed_upload_is_made_up_for(fake):
+    """After a copy that failed, the next step uploads the counts again."""
+    s = lbfs.Solver(precision=lbfs.FP64, max_cases=2)
+    for k in range(2):
+        s.set_case(k, _case())
+    for n in range(1, 4):
+        fake.set("failing_copies", n)
+        status, _ = s.step(1, raise_on_error=False)
+        assert status in (lbfs.ECUDA, lbfs.ENOMEM)
+    fake.set("failing_copies", 0)
+    fake.clear()
+    s.step(1)
+    s.close()
+    stages = [w for w in fake.log() if w[0] == "stage"]
+    assert len(stages) == 3 and all(w[2:] == ["batch"] for w in stages), stages
