@@ -16,7 +16,6 @@ using namespace lbfs;
 namespace {
 
 constexpr int kCoarsenCells = 4;      // stop coarsening at or below this many cells
-constexpr int kCoarsestMax = 4096;    // largest coarsest level accepted
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -655,7 +654,10 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
         cudaGetLastError();
         return LBFS_ECUDA;
     }
-    if (cudaSetDevice(cfg->device) != cudaSuccess) return LBFS_ECUDA;
+    if (cudaSetDevice(cfg->device) != cudaSuccess || prepare_potential(cfg->precision) != cudaSuccess) {
+        cudaGetLastError();
+        return LBFS_ECUDA;
+    }
     lbfs_ctx* ctx = new lbfs_ctx();
     ctx->cfg = *cfg;
     ctx->prec = cfg->precision;

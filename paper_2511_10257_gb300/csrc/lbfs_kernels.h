@@ -46,6 +46,9 @@ cudaError_t launch_pseudo_time(int prec, const DevCase* dcase, int nx, int ny, i
 // The V-cycle's levels from DevCase::tail down, one block per case.  A case takes it when its
 // coarsest level holds at most kTailCoarsest cells, from the first level of at most kTailCells.
 constexpr int kTailCells = 2048, kTailCoarsest = 1024, kPassCells = 256;
+constexpr int kCoarsestMax = 4096;    // largest coarsest level accepted
+// once on a context's device, before the launches below: their kernels' shared-memory limits
+cudaError_t prepare_potential(int prec);
 cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* case_ids, int ncases, int max_cells, int max_small,
                            cudaStream_t st);
 // the coarsest level of the other cases

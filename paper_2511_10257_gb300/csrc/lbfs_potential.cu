@@ -1466,8 +1466,30 @@ cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, 
     return cudaGetLastError();
 }
 
-static size_t tail_bytes(int max_cells, int max_small) {
+static constexpr size_t tail_bytes(int max_cells, int max_small) {
     return ((size_t)8 * max_cells + (size_t)2 * max_small) * sizeof(float);
+}
+static constexpr size_t coarsest_bytes(int max_cells) { return (size_t)5 * max_cells * sizeof(float); }
+
+// The dynamic shared memory a kernel may ask for belongs to the kernel on its device, not to a
+// context or a launch, and other threads' contexts launch the same kernels: it is set to what the
+// largest cases need (a level has at most 9/25 of the cells above it, so a tail fewer than twice
+// its first level's), always the same, and never by a step.
+constexpr size_t kTailLimit = tail_bytes(2 * kTailCells, kTailCoarsest), kCoarsestLimit = coarsest_bytes(kCoarsestMax);
+constexpr size_t kCyclesLimit =
+    std::max({(size_t)kLegGroups * kLegBytes<kFusedTX, kFusedTY>, kTailLimit, kCoarsestLimit});
+static_assert(kCyclesLimit <= 220 * 1024, "leaves the static shared memory its place in a block's 227 KB");
+
+cudaError_t prepare_potential(int prec) {
+    const auto limit = [](const void* kern, size_t bytes) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    const void* tail = prec == 0 ? (const void*)k_tail<double> : (const void*)k_tail<float>;
+    const void* cycles = prec == 0 ? (const void*)k_cycles<double> : (const void*)k_cycles<float>;
+    cudaError_t e = limit(tail, kTailLimit);
+    if (e == cudaSuccess) e = limit((const void*)k_coarsest, kCoarsestLimit);
+    if (e == cudaSuccess) e = limit(cycles, kCyclesLimit);
+    return e;
 }
 
 cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* ids, int ncases, int max_cells, int max_small,
@@ -1475,28 +1497,21 @@ cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* ids, int n
     if (ncases <= 0) return cudaSuccess;
     const size_t sm = tail_bytes(max_cells, max_small);
     auto kern = prec == 0 ? k_tail<double> : k_tail<float>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     kern<<<ncases, kTailNT, sm, st>>>(cases, ids, max_cells, max_small);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mg_coarsest(const DevCase* cases, const int* ids, int ncases, int max_cells, cudaStream_t st) {
     if (ncases <= 0) return cudaSuccess;
-    const size_t sm = (size_t)5 * max_cells * sizeof(float);
-    const cudaError_t e = cudaFuncSetAttribute(k_coarsest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    k_coarsest<<<ncases, kTailNT, sm, st>>>(cases, ids);
+    k_coarsest<<<ncases, kTailNT, coarsest_bytes(max_cells), st>>>(cases, ids);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mg_cycles(int prec, const CycleArgs& a, int blocks, int max_coarsest, const PotCheck& ck,
                              cudaStream_t st) {
     const size_t sm = std::max({(size_t)kLegGroups * kLegBytes<kFusedTX, kFusedTY>, tail_bytes(a.tail_cells, a.tail_small),
-                                (size_t)5 * max_coarsest * sizeof(float)});
+                                coarsest_bytes(max_coarsest)});
     auto kern = prec == 0 ? k_cycles<double> : k_cycles<float>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     void* args[] = {const_cast<CycleArgs*>(&a), const_cast<PotCheck*>(&ck)};
     return cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(kTailNT), args, sm, st);
 }

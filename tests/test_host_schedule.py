@@ -110,3 +110,27 @@ def test_a_failed_upload_is_made_up_for(fake):
     s.close()
     stages = [w for w in fake.log() if w[0] == "stage"]
     assert len(stages) == 3 and all(w[2:] == ["batch"] for w in stages), stages
+
+
+@pytest.mark.parametrize("precision", BOTH)
+def test_a_step_changes_no_limit_of_a_kernel(fake, precision):
+    """A kernel's shared-memory limit is the whole process's: a context of small cases, stepped by
+    another thread between a larger one's set-up of the limit and its launch, must not lower it."""
+    large = [_case(91, 45), _case(126, 64, periodic_x=1), _case(6, 2700, periodic_x=1)]   # coarsest 4050 cells
+    small = [_case(8, 8)]
+    solvers = []
+    for cases in (large, small):
+        s = lbfs.Solver(precision=precision, max_cases=len(cases), mg_plain_cycles=len(solvers) == 1)
+        for k, c in enumerate(cases):
+            s.set_case(k, c)
+        solvers.append(s)
+    fake.clear()
+    for _ in range(2):
+        for s in solvers:
+            s.step(2)
+    for s in solvers:
+        s.close()
+    log = fake.log()
+    assert not [w for w in log if w[0] == "limit"]
+    sizes = [(int(w[6]), int(w[8])) for w in log if w[0] in ("launch", "cooperative")]
+    assert max(n for n, _ in sizes) > 48 * 1024 and all(n <= limit for n, limit in sizes)
