@@ -79,7 +79,10 @@ typedef struct lbfs_config {
                                 after a state is set are counted on the host), instead of
                                 one cooperative kernel for the last of them (a profiler
                                 shows their phases); same results                         */
-    int32_t reserved[5];
+    int32_t mg_wait_polls;   /* polls after which a wait between the blocks of that kernel gives
+                                up and lbfs_step returns LBFS_ETIMEOUT (0: 2^22, seconds); the
+                                blocks run at the same time, so it is not met in practice   */
+    int32_t reserved[4];
 } lbfs_config;
 
 /* One case.  Walls are numbered 0 left (x = 0), 1 right (x = nx), 2 bottom (y = 0),
@@ -186,7 +189,9 @@ lbfs_status lbfs_set_fields(lbfs_ctx* ctx, int32_t case_id, uint32_t mask, const
  * statistics.  Runs on the context's stream and waits for completion.  out (nullable,
  * caller-owned, max_cases entries) receives each slot's statistics (undefined slots
  * zero).  nsteps < 0 gives LBFS_EINVAL before any launch; LBFS_EDIVERGED (a non-finite
- * value) and LBFS_ENOTCONVERGED (the potential missed its tolerance) are reported after
+ * value), LBFS_ENOTCONVERGED (the potential missed its tolerance) and LBFS_ETIMEOUT (a wait
+ * on the device ran out of mg_wait_polls with the potential unsolved; the state is that of
+ * steps with an unsolved potential, and the next call solves it afresh) are reported after
  * the steps ran, with the stats still filled. */
 lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out);
 

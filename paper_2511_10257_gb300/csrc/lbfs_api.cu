@@ -17,6 +17,8 @@ namespace {
 
 constexpr int kCoarsenCells = 4;      // stop coarsening at or below this many cells
 
+constexpr int kFlags = 4;             // words of lbfs_ctx::d_flag
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Slot {
@@ -26,6 +28,7 @@ struct Slot {
     StageCase<float> sf{};    // the stage kernel's view, in the context's precision
     StageCase<double> sd{};
     void* block = nullptr;
+    size_t ticket_bytes = 0;  // of hd.mg_tickets
 };
 
 }  // namespace
@@ -56,7 +59,10 @@ struct lbfs_ctx {
     int n_coarsest = 0, coarsest_cells = 0;
     int max_depth = 0;                  // levels with a kernel per leg
     int sm_count = 152;               // multiprocessors of the context's device
+    // after the statistics, copied to the host with them: [0] votes of host-counted cycles, [1] and
+    // [2] the cycles' grid barrier, [3] a wait in it ran out
     int* d_flag = nullptr;
+    size_t stats_bytes = 0;   // of the statistics, to the flags
     int* h_flag = nullptr;
     double* h_stats = nullptr;
     double* d_scratch = nullptr;
@@ -68,6 +74,7 @@ struct lbfs_ctx {
     double mg_tol = 0.0;
     int mg_max_cycles = 0;
     int mg_warm_cycles = 0;
+    int mg_wait_polls = 0;
     int half = 0;          // every defined case has dts = 1/2
     int tile = 0;          // stage-kernel strip shape id (config or autotuner)
     int rows = 0;          // rows of a strip, by the shape id or its rule
@@ -483,7 +490,7 @@ lbfs_status vcycle(lbfs_ctx* ctx) {
 }
 
 PotCheck pot_check(const lbfs_ctx* ctx, int first, int kmax, int* not_done) {
-    return PotCheck{first, ctx->mg_tol, kmax, not_done, reinterpret_cast<unsigned*>(ctx->d_flag + 1)};
+    return PotCheck{first, ctx->mg_tol, kmax, not_done, reinterpret_cast<unsigned*>(ctx->d_flag + 1), ctx->mg_wait_polls};
 }
 
 // the residual of the master potential and each case's check
@@ -664,6 +671,7 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
     ctx->mg_tol = cfg->mg_tol > 0 ? cfg->mg_tol : (ctx->prec == 0 ? 1e-13 : 1e-6);
     ctx->mg_max_cycles = cfg->mg_max_cycles > 0 ? cfg->mg_max_cycles : 40;
     ctx->mg_warm_cycles = cfg->mg_warm_cycles > 0 ? cfg->mg_warm_cycles : (ctx->prec == 0 ? 12 : 3);
+    ctx->mg_wait_polls = cfg->mg_wait_polls > 0 ? cfg->mg_wait_polls : kWaitPolls;
     ctx->slots.resize(cfg->max_cases);
     ctx->tile = (cfg->tile >= 0 && cfg->tile < stage_tile_shapes()) ? cfg->tile : 0;
     {
@@ -695,11 +703,12 @@ lbfs_status lbfs_create(const lbfs_config* cfg, lbfs_ctx** out) {
     }
     if (!ctx->d_cases ||
         cudaMallocHost(&ctx->h_flag, sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_stats, sizeof(double) * kStatN * cfg->max_cases) != cudaSuccess) {
+        cudaMallocHost(&ctx->h_stats, stats_b + kFlags * sizeof(int)) != cudaSuccess) {
         lbfs_destroy(ctx);
         return LBFS_ENOMEM;
     }
-    cudaMemset(ctx->d_cases, 0, cases_b + stage_b + stats_b + 256);   // d_flag: [0] host-checked votes, [1] and [2] the cycles' grid barrier
+    ctx->stats_bytes = stats_b;
+    cudaMemset(ctx->d_cases, 0, cases_b + stage_b + stats_b + 256);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         lbfs_destroy(ctx);
         return LBFS_ECUDA;
@@ -796,7 +805,8 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     add((void**)&hd.red_tickets, (size_t)(1 + red_groups) * sizeof(unsigned));
     add((void**)&hd.mg_red, (size_t)res_cap * 2 * sizeof(double));
     add((void**)&hd.mg_groups, (size_t)res_groups * 2 * sizeof(double));
-    add((void**)&hd.mg_tickets, (size_t)(1 + res_groups) * sizeof(unsigned));
+    const size_t ticket_bytes = (size_t)(1 + res_groups) * sizeof(unsigned);
+    add((void**)&hd.mg_tickets, ticket_bytes);
     add((void**)&hd.chunk, (size_t)kFinChunks * kRedN * sizeof(double));
     add((void**)&hd.tickets, sizeof(unsigned));
     Slot& s = ctx->slots[id];
@@ -811,6 +821,7 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     if (ctx->prec == 0) hd.phi = hd.phi64;
     hd.stats = ctx->d_stats + (size_t)id * kStatN;
     s.hd = hd;
+    s.ticket_bytes = ticket_bytes;
     s.desc = *desc;
     const void* sc = &s.sf;
     size_t scb = sizeof(s.sf);
@@ -970,10 +981,18 @@ lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
         lbfs_status r = one_step(ctx);
         if (r != LBFS_OK) return r;
     }
-    const size_t nb = sizeof(double) * kStatN * ctx->slots.size();
-    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, nb, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, ctx->stats_bytes + kFlags * sizeof(int), cudaMemcpyDeviceToHost,
+                       ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     harvest(ctx);
+    const bool timed_out = reinterpret_cast<const int*>(reinterpret_cast<const char*>(ctx->h_stats) + ctx->stats_bytes)[3] != 0;
+    if (timed_out) {   // blocks left the cycles at different places: no ticket keeps a count, the next step solves afresh
+        for (const Slot& s : ctx->slots)
+            if (s.defined) CK(cudaMemsetAsync(s.hd.mg_tickets, 0, s.ticket_bytes, ctx->stream));
+        CK(cudaMemsetAsync(ctx->d_flag, 0, kFlags * sizeof(int), ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        ctx->pot_fresh = true;
+    }
     bool bad = false;
     for (size_t c = 0; c < ctx->slots.size(); ++c) {
         const double* st = ctx->h_stats + c * kStatN;
@@ -997,6 +1016,8 @@ lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
             o.pot_cycles_mean = st[ST_STEPS_CALL] > 0 ? st[ST_POT_CYCLES_SUM] / st[ST_STEPS_CALL] : 0.0;
         }
     }
+    if (timed_out)
+        return fail(ctx, LBFS_ETIMEOUT, "a wait between the blocks of the potential's cycles ran out of its polls (mg_wait_polls)");
     if (bad) return fail(ctx, LBFS_EDIVERGED, "a non-finite value appeared in a case's state");
     if (ctx->pot_fail)
         return fail(ctx, LBFS_ENOTCONVERGED,

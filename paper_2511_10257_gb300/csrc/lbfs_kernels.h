@@ -28,7 +28,8 @@ constexpr int kMgTX = 32, kMgTY = 32;
 // each case once its strips are done.  first: the step's first residual (every case; later ones
 // skip converged cases).  tol: the convergence test.  A case still above tol gets another cycle
 // (one more vote in not_done, if given) unless it has had kmax, when it is marked as failed.
-// sync: the grid barrier of launch_mg_cycles (two counters), cleared by a first check.
+// sync: the grid barrier of launch_mg_cycles: two counters, cleared by a first check, and a mark
+// that a wait of more than wait_polls polls ran out, cleared by the host.
 constexpr int kResidStripW = 30, kResidMinRows = 2;
 struct PotCheck {
     int first;
@@ -36,6 +37,7 @@ struct PotCheck {
     int kmax;
     int* not_done;
     unsigned* sync;
+    int wait_polls;
 };
 cudaError_t launch_mg_residual(int prec, const DevCase* cases, const TileRef* tiles, int n, int rows, const PotCheck& ck,
                                cudaStream_t st);
@@ -63,6 +65,7 @@ cudaError_t launch_mg_vdown(int prec, const DevCase* cases, const TileRef* tiles
                             cudaStream_t st);
 cudaError_t launch_mg_vup(int prec, const DevCase* cases, const TileRef* tiles, int n, int level, int small,
                           cudaStream_t st);
+constexpr int kWaitPolls = 1 << 22;   // default limit of a grid barrier's wait: seconds
 // Cycles (V-cycle, residual, check) until no case needs another, in one cooperative launch of
 // `blocks` blocks (at most one an SM), after a first launch_mg_residual with the same check
 // and first set to 0.  max_coarsest: as for launch_mg_coarsest, 0 without such a case.

@@ -1188,17 +1188,15 @@ constexpr int kLegNT = 256, kLegGroups = kTailNT / kLegNT;
 
 // All blocks of the grid arrive (sync[0] counts them; it starts a launch at zero and only
 // grows).  The blocks of a cooperative launch run at the same time, so the wait ends; should it
-// not within kSyncPolls polls (seconds), sync[1] tells every block to give up.
-constexpr int kSyncPolls = 1 << 22;
-
-__device__ __forceinline__ bool grid_sync(unsigned* sync, unsigned& target, int* ok) {
+// not within `limit` polls, sync[1] tells every block to give up.
+__device__ __forceinline__ bool grid_sync(unsigned* sync, unsigned& target, int limit, int* ok) {
     target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(sync, 1u);
         int polls = 0;
-        while (*static_cast<volatile unsigned*>(sync) < target && ++polls < kSyncPolls &&
+        while (*static_cast<volatile unsigned*>(sync) < target && ++polls < limit &&
                *static_cast<volatile unsigned*>(sync + 1) == 0u) {
         }
         __threadfence();
@@ -1245,14 +1243,14 @@ __global__ void __launch_bounds__(kTailNT, 1) k_cycles(const __grid_constant__ C
                 }
                 sync();   // the tile's memory is free again
             }
-            alive = grid_sync(ck.sync, target, &ok);
+            alive = grid_sync(ck.sync, target, ck.wait_polls, &ok);
         }
         for (int q = b; q < cases_n && alive; q += nb) {
             if (q < a.n_tail) tail_case<M0>(case_of(q), a.tail_cells, a.tail_small, mem, lv, geo);
             else coarsest_case(case_of(q), mem, red);
             __syncthreads();
         }
-        alive = alive && grid_sync(ck.sync, target, &ok);
+        alive = alive && grid_sync(ck.sync, target, ck.wait_polls, &ok);
         for (int L = a.depth - 1; L >= 0 && alive; --L) {
             for (int t = group * nb + b; t < a.n_tiles[L]; t += kLegGroups * nb) {
                 const TileRef tr = a.tiles[L][t];
@@ -1266,18 +1264,17 @@ __global__ void __launch_bounds__(kTailNT, 1) k_cycles(const __grid_constant__ C
                 }
                 sync();
             }
-            alive = grid_sync(ck.sync, target, &ok);
+            alive = grid_sync(ck.sync, target, ck.wait_polls, &ok);
         }
         if (alive) {
             for (int t = (threadIdx.x >> 5) * nb + b; t < a.n_strips; t += (kTailNT >> 5) * nb) {
                 const TileRef tr = a.strips[t];
                 residual_strip<M0>(a.cases + tr.case_id, tr, a.rows, ck, threadIdx.x & 31);
             }
-            alive = grid_sync(ck.sync, target, &ok);
+            alive = grid_sync(ck.sync, target, ck.wait_polls, &ok);
         }
-        if (!alive) {   // reported as a potential that has not converged
-            for (int q = threadIdx.x; q < cases_n; q += kTailNT)
-                if (!pot_done(case_of(q))) case_of(q)->stats[ST_POT_FAIL] = 1.0;
+        if (!alive) {   // the host reports it and clears the tickets of a residual some blocks did not take
+            if (threadIdx.x == 0) atomicExch(ck.sync + 2, 1u);
             return;
         }
         more = pending();

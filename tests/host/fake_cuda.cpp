@@ -119,7 +119,9 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int v) {
     g_attr[f] = v;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3 grid, dim3, void**, size_t smem, cudaStream_t s) {
+void fake_cycles(void** args, cudaStream_t s, int runs_out);
+cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3 grid, dim3, void** args, size_t smem, cudaStream_t s) {
+    fake_cycles(args, s, (int)g_set["wait_runs_out"]);
     return launched(f, grid, smem, s, "cooperative");
 }
 

@@ -134,3 +134,25 @@ def test_a_step_changes_no_limit_of_a_kernel(fake, precision):
     assert not [w for w in log if w[0] == "limit"]
     sizes = [(int(w[6]), int(w[8])) for w in log if w[0] in ("launch", "cooperative")]
     assert max(n for n, _ in sizes) > 48 * 1024 and all(n <= limit for n, limit in sizes)
+
+
+@pytest.mark.parametrize("precision", BOTH)
+@pytest.mark.parametrize("graph", [False, True])
+def test_a_wait_that_ran_out_is_reported_as_such(fake, precision, graph):
+    """LBFS_ETIMEOUT, not a potential that has not converged; the counts that the blocks left
+    behind are cleared, and the next step solves the potential afresh."""
+    s = lbfs.Solver(precision=precision, max_cases=2, use_graph=graph)
+    for k in range(2):
+        s.set_case(k, _case(300, 150))
+    s.step(2)
+    fake.set("wait_runs_out", 1)
+    s.set_case(1, _case(300, 150))
+    status, _ = s.step(1, raise_on_error=False)
+    fake.set("wait_runs_out", 0)
+    fake.clear()
+    again, _ = s.step(1, raise_on_error=False)
+    s.close()
+    log = fake.log()
+    assert status == lbfs.ETIMEOUT and again == lbfs.OK
+    assert [w[2] for w in log if w[0] == "ticket"] == ["0"]
+    assert [w[0] for w in log if w[0] in ("cooperative", "replay")] == ["cooperative"]
