@@ -78,7 +78,9 @@ typedef struct lbfs_config {
                                 kernels, each returning at once for a converged case (those
                                 after a state is set are counted on the host), instead of
                                 one cooperative kernel for the last of them (a profiler
-                                shows their phases); same results                         */
+                                shows their phases); same results.  So are they where that
+                                kernel cannot run, on a stream with a part of the device's
+                                multiprocessors                                            */
     int32_t mg_wait_polls;   /* polls after which a wait between the blocks of that kernel gives
                                 up and lbfs_step returns LBFS_ETIMEOUT (0: 2^22, seconds); the
                                 blocks run at the same time, so it is not met in practice   */
@@ -191,7 +193,8 @@ lbfs_status lbfs_set_fields(lbfs_ctx* ctx, int32_t case_id, uint32_t mask, const
  * zero).  nsteps < 0 gives LBFS_EINVAL before any launch; LBFS_EDIVERGED (a non-finite
  * value), LBFS_ENOTCONVERGED (the potential missed its tolerance) and LBFS_ETIMEOUT (a wait
  * on the device ran out of mg_wait_polls with the potential unsolved; the state is that of
- * steps with an unsolved potential, and the next call solves it afresh) are reported after
+ * steps with an unsolved potential, and the next call solves it afresh, with launched
+ * cycles) are reported after
  * the steps ran, with the stats still filled. */
 lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out);
 

@@ -79,6 +79,9 @@ struct lbfs_ctx {
     int tile = 0;          // stage-kernel strip shape id (config or autotuner)
     int rows = 0;          // rows of a strip, by the shape id or its rule
     bool pot_fresh = true; // a state was set since the last full potential solve
+    // whether all blocks of the cycles' kernel run at once on the context's stream: -1 not known
+    // yet, 1 it has run, 0 it was refused or a wait of its ran out
+    int coop = -1;
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
     int64_t graph_launches = 0;       // kernel nodes in one recorded step
@@ -536,6 +539,10 @@ int phased_cycles(int prec, int cases) {
     return prec == 0 ? 4 : (cases >= 4 ? 1 : 0);
 }
 
+// whether all cycles are launched phase by phase: as configured, or because the kernel that takes
+// them in one launch needs all its blocks to run at once and cannot have that on this stream
+bool launched_cycles(const lbfs_ctx* ctx) { return ctx->cfg.mg_plain_cycles || ctx->coop == 0; }
+
 // The potential of the current state: in FP64 a warm step starts from the linearly
 // extrapolated potential; then the step's first residual and check, then refinement cycles
 // (V-cycle, correction, residual of the corrected potential, check), which the checks end on the
@@ -549,7 +556,8 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
     cudaStream_t s = ctx->stream;
     if (ctx->prec == 0 && !ctx->pot_fresh)
         LK(launch_mg_extrapolate(ctx->d_cases, ctx->d_mg_tiles, ctx->n_mg_tiles, s));
-    if (ctx->cfg.mg_plain_cycles && ctx->pot_fresh) {   // as many as are needed, counted on the host
+    const bool launched = launched_cycles(ctx);
+    if (launched && ctx->pot_fresh) {   // as many as are needed, counted on the host
         for (int it = 0;; ++it) {
             CK(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s));
             LK(check_residual(ctx, it == 0, kmax, ctx->d_flag));
@@ -560,14 +568,23 @@ lbfs_status potential_solve(lbfs_ctx* ctx) {
             if (r != LBFS_OK) return r;
         }
     } else {
-        const int phased = ctx->cfg.mg_plain_cycles ? kmax : std::min(kmax, phased_cycles(ctx->prec, ctx->n_pot));
+        const int phased = launched ? kmax : std::min(kmax, phased_cycles(ctx->prec, ctx->n_pot));
         LK(check_residual(ctx, 1, kmax, nullptr));
-        for (int c = 0; c < phased; ++c) {
+        for (int c = 0; c < kmax; ++c) {
+            if (c == phased) {
+                const cudaError_t e = cycles(ctx, kmax);
+                if (e != cudaErrorCooperativeLaunchTooLarge) {
+                    LK(e);
+                    ctx->coop = 1;
+                    break;
+                }
+                cudaGetLastError();   // the stream has fewer multiprocessors than the device: launch the rest
+                ctx->coop = 0;
+            }
             lbfs_status r = vcycle(ctx);
             if (r != LBFS_OK) return r;
             LK(check_residual(ctx, 0, kmax, nullptr));
         }
-        if (phased < kmax) LK(cycles(ctx, kmax));
     }
     if (ctx->pot_fresh) {
         // the warm steps that follow extrapolate only once they have stored a potential
@@ -968,7 +985,9 @@ lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
         }
     for (int n = 0; n < nsteps && ctx->n_active > 0; ++n) {
         // a step after the first potential solve has no host round trip and can be replayed
-        const bool graphable = ctx->cfg.use_graph && !ctx->timing && !(ctx->n_pot > 0 && ctx->pot_fresh);
+        // (not before it is known whether the cycles' kernel can run: a refusal would end the recording)
+        const bool known = launched_cycles(ctx) || ctx->coop == 1 || phased_cycles(ctx->prec, ctx->n_pot) >= ctx->mg_warm_cycles;
+        const bool graphable = ctx->cfg.use_graph && !ctx->timing && !(ctx->n_pot > 0 && (ctx->pot_fresh || !known));
         if (graphable) {
             if (!ctx->gexec) {
                 lbfs_status r = record_graph(ctx);
@@ -986,12 +1005,15 @@ lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
     CK(cudaStreamSynchronize(ctx->stream));
     harvest(ctx);
     const bool timed_out = reinterpret_cast<const int*>(reinterpret_cast<const char*>(ctx->h_stats) + ctx->stats_bytes)[3] != 0;
-    if (timed_out) {   // blocks left the cycles at different places: no ticket keeps a count, the next step solves afresh
+    if (timed_out) {   // blocks left the cycles at different places: no ticket keeps a count, the next step solves afresh,
+                       // with launched cycles
         for (const Slot& s : ctx->slots)
             if (s.defined) CK(cudaMemsetAsync(s.hd.mg_tickets, 0, s.ticket_bytes, ctx->stream));
         CK(cudaMemsetAsync(ctx->d_flag, 0, kFlags * sizeof(int), ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         ctx->pot_fresh = true;
+        ctx->coop = 0;
+        drop_graph(ctx);
     }
     bool bad = false;
     for (size_t c = 0; c < ctx->slots.size(); ++c) {

@@ -10,14 +10,16 @@
 extern "C" void fake_say(const char* what, cudaStream_t s, const char* more);
 
 // What the cycles' kernel leaves behind when its grid barrier runs out: the mark, and a ticket of
-// a residual that not every block has taken.  Notes the ticket it finds.
-extern "C" void fake_cycles(void** args, cudaStream_t s, int runs_out) {
+// a residual that not every block has taken.
+extern "C" void fake_cycles(void** args) {
     const lbfs::CycleArgs& a = *static_cast<const lbfs::CycleArgs*>(args[0]);
     const lbfs::PotCheck& ck = *static_cast<const lbfs::PotCheck*>(args[1]);
-    fake_say("ticket", s, std::to_string(a.cases[0].mg_tickets[1]).c_str());
-    if (!runs_out) return;
     a.cases[0].mg_tickets[1] = 7;
     ck.sync[1] = ck.sync[2] = 1;
+}
+// a residual: the ticket it finds
+extern "C" void fake_residual(void** args, cudaStream_t s) {
+    fake_say("ticket", s, std::to_string((*static_cast<const lbfs::DevCase**>(args[0]))->mg_tickets[1]).c_str());
 }
 
 namespace lbfs {

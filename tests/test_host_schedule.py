@@ -151,8 +151,43 @@ def test_a_wait_that_ran_out_is_reported_as_such(fake, precision, graph):
     fake.set("wait_runs_out", 0)
     fake.clear()
     again, _ = s.step(1, raise_on_error=False)
+    third, _ = s.step(1, raise_on_error=False)
     s.close()
     log = fake.log()
-    assert status == lbfs.ETIMEOUT and again == lbfs.OK
-    assert [w[2] for w in log if w[0] == "ticket"] == ["0"]
-    assert [w[0] for w in log if w[0] in ("cooperative", "replay")] == ["cooperative"]
+    assert status == lbfs.ETIMEOUT and again == third == lbfs.OK
+    assert not [w for w in log if w[0] == "cooperative"]   # launched from now on
+    assert [w[0] for w in log].count("replay") == (1 if graph else 0)
+    assert {w[2] for w in log if w[0] == "ticket"} == {"0"}
+
+
+@pytest.mark.parametrize("precision", BOTH)
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("first", [1, 40])   # cycles of the first solve: fewer and more than are launched anyway
+def test_a_refused_cooperative_launch_falls_back(fake, precision, graph, first):
+    """On a stream with fewer multiprocessors than the device has, the cycles are launched phase by
+    phase, as many as the kernel would have run; the refused launch is not tried again and never
+    part of a recording."""
+    s = lbfs.Solver(precision=precision, max_cases=2, use_graph=graph, mg_max_cycles=first)
+    for k in range(2):
+        s.set_case(k, _case(300, 150))
+    fake.set("cooperative_limit", 2)
+    fake.clear()
+    s.step(3)
+    log = fake.log()
+    kinds = [w[0] for w in log]
+    assert kinds.count("refused") == 1 and "cooperative" not in kinds
+    if graph:
+        assert kinds.index("refused") < kinds.index("record")
+    fake.clear()
+    s.set_case(1, _case(300, 150))   # a new recording
+    s.step(3)
+    s.close()
+    fake.set("cooperative_limit", 1 << 20)
+    log = fake.log()
+    assert not [w for w in log if w[0] in ("refused", "cooperative")]
+    tails = [k for k, w in enumerate(log) if w[0] == "launch" and w[2].startswith("k_tail")]
+    if graph:   # one recorded warm step: its checks are of the step's start and after each cycle
+        a, b = [[w[0] for w in log].index(x) for x in ("record", "recorded")]
+        checks = [k for k, w in enumerate(log) if w[0] == "launch" and w[2].startswith("k_residual") and a < k < b]
+        warm = 12 if precision == lbfs.FP64 else 3
+        assert len(checks) == warm + 1 and sum(a < k < b for k in tails) == warm
