@@ -59,7 +59,7 @@ typedef struct lbfs_config {
     void* (*dev_alloc)(size_t bytes, void* user);  /* optional device allocator, e.g. a   */
     void  (*dev_free)(void* ptr, void* user);      /* framework's caching allocator; the
                                 memory is used on cuda_stream at once, so no other stream
-                                may have work left on it                                   */
+                                may have work left on it; alignment: 8 bytes at least      */
     void*   alloc_user;
     int32_t mg_max_cycles;   /* refinement cycles of a potential solve after a state is set,
                                 checked on the device (0: 40)                              */

@@ -17,6 +17,8 @@ namespace {
 
 constexpr int kCoarsenCells = 4;      // stop coarsening at or below this many cells
 
+constexpr size_t kFieldAlign = 32;    // of a case's arrays: one load of a cell's four FP64 quantities
+static_assert(kFieldAlign % alignof(Quad64) == 0, "a case's quads lie on their own boundary");
 constexpr int kFlags = 4;             // words of lbfs_ctx::d_flag
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -830,9 +832,12 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     free_slot(ctx, s);
     drop_graph(ctx);
     ctx->dirty = true;
-    s.block = dalloc(ctx, off);
+    // cudaMalloc aligns to 256 bytes; an allocator of the caller's to 8 at least, from where the
+    // arrays are moved up to the next multiple of a field's widest load
+    s.block = dalloc(ctx, off + (ctx->cfg.dev_alloc ? kFieldAlign : 0));
     if (!s.block) return fail(ctx, LBFS_ENOMEM, "device allocation of the case failed");
-    for (auto& pr : plan) *pr.first = static_cast<char*>(s.block) + pr.second;
+    char* base = reinterpret_cast<char*>(align_up(reinterpret_cast<size_t>(s.block), kFieldAlign));
+    for (auto& pr : plan) *pr.first = base + pr.second;
     for (int L = 0; L < nlev; ++L)
         if (!hd.lev[L].eu) hd.lev[L].eu = hd.lev[L].e;
     if (ctx->prec == 0) hd.phi = hd.phi64;
@@ -849,7 +854,7 @@ lbfs_status lbfs_set_case(lbfs_ctx* ctx, int32_t id, const lbfs_case_desc* desc)
     } else {
         fill_stage<float>(hd, s.sf);
     }
-    CK(cudaMemsetAsync(s.block, 0, off, ctx->stream));
+    CK(cudaMemsetAsync(base, 0, off, ctx->stream));
     CK(cudaMemcpyAsync(ctx->d_cases + id, &s.hd, sizeof(DevCase), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(static_cast<char*>(ctx->d_stage_cases) + id * scb, sc, scb, cudaMemcpyHostToDevice, ctx->stream));
     double st0[kStatN];

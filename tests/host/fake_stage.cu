@@ -24,12 +24,20 @@ extern "C" void fake_residual(void** args, cudaStream_t s) {
 
 namespace lbfs {
 
+template <class R>
+std::string misplaced(const StageCase<R>& c) {
+    for (const void* p : {c.He[0], c.He[1], c.He[2], c.W[0], c.W[1], c.W[2], c.phi, c.Fs_prev, c.Sdot, c.mu})
+        if (reinterpret_cast<size_t>(p) % 32) return " misplaced";
+    return "";
+}
 template <class R, bool HALF, bool UNI>
-cudaError_t stage_launch(const StageCase<R>&, const StageCase<R>* cases, const TileRef* tiles, int ntiles, int, int,
+cudaError_t stage_launch(const StageCase<R>& one, const StageCase<R>* cases, const TileRef* tiles, int ntiles, int, int,
                          cudaStream_t st) {
     std::map<int, int> n;
     for (int t = 0; t < ntiles; ++t) ++n[tiles[t].case_id];
-    std::string more = UNI ? "one" : "batch";
+    std::string more = UNI ? "one" + misplaced(one) : "batch";
+    for (const auto& c : n)
+        if (!UNI) more += misplaced(cases[c.first]);
     for (const auto& c : n)
         if (!UNI && cases[c.first].strips != c.second)
             more += " case " + std::to_string(c.first) + ": " + std::to_string(cases[c.first].strips) + " strips of " +

@@ -28,12 +28,13 @@ def _case(nx=64, ny=32, **kw):
     return I.case(nx, ny, radius=9.0, H0=0.03, field_angle_deg=40.0, **kw)
 
 
-def test_torch_memory_is_free_of_pending_work_before_it_is_used(fake, monkeypatch):
-    """A block of torch's caching allocator may still be in use by kernels queued on torch's
-    current stream; the library's stream is not ordered behind them."""
+def _torch_memory(monkeypatch, offset=0):
+    """torch's caching allocator over the host's memory, `offset` bytes past a multiple of 64; the
+    list of its calls"""
     torch = pytest.importorskip("torch")
     libc = ct.CDLL(None)
-    libc.malloc.restype, libc.malloc.argtypes, libc.free.argtypes = ct.c_void_p, [ct.c_size_t], [ct.c_void_p]
+    libc.aligned_alloc.restype, libc.aligned_alloc.argtypes = ct.c_void_p, [ct.c_size_t, ct.c_size_t]
+    libc.free.argtypes = [ct.c_void_p]
     calls = []
 
     class Stream:
@@ -42,11 +43,18 @@ def test_torch_memory_is_free_of_pending_work_before_it_is_used(fake, monkeypatc
 
     def alloc(n, device):
         calls.append("allocated")
-        return libc.malloc(n)
+        return libc.aligned_alloc(64, (n + 127) // 64 * 64) + offset
 
     monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", alloc)
-    monkeypatch.setattr(torch.cuda, "caching_allocator_delete", libc.free)
+    monkeypatch.setattr(torch.cuda, "caching_allocator_delete", lambda p: libc.free(p - offset))
     monkeypatch.setattr(torch.cuda, "current_stream", lambda device: Stream())
+    return calls
+
+
+def test_torch_memory_is_free_of_pending_work_before_it_is_used(fake, monkeypatch):
+    """A block of torch's caching allocator may still be in use by kernels queued on torch's
+    current stream; the library's stream is not ordered behind them."""
+    calls = _torch_memory(monkeypatch)
     s = lbfs.Solver(precision=lbfs.MIXED, max_cases=1, torch_alloc=True)
     s.set_case(0, _case())
     s.step(1)
@@ -191,3 +199,19 @@ def test_a_refused_cooperative_launch_falls_back(fake, precision, graph, first):
         checks = [k for k, w in enumerate(log) if w[0] == "launch" and w[2].startswith("k_residual") and a < k < b]
         warm = 12 if precision == lbfs.FP64 else 3
         assert len(checks) == warm + 1 and sum(a < k < b for k in tails) == warm
+
+
+@pytest.mark.parametrize("precision", BOTH)
+@pytest.mark.parametrize("offset", [0, 8, 24, 40])
+def test_a_callers_allocator_need_not_align_to_a_quad(fake, monkeypatch, precision, offset):
+    """The kernels read a cell's quantities 16 and 32 bytes at a time."""
+    _torch_memory(monkeypatch, offset)
+    for cases in (1, 2):
+        s = lbfs.Solver(precision=precision, max_cases=cases, torch_alloc=True)
+        for k in range(cases):
+            s.set_case(k, _case())
+        fake.clear()
+        s.step(1)
+        s.close()
+        stages = [w for w in fake.log() if w[0] == "stage"]
+        assert len(stages) == 3 and not [w for w in stages if "misplaced" in w]
