@@ -975,11 +975,11 @@ lbfs_status lbfs_potential_pseudo_time(lbfs_ctx* ctx, int32_t id, int32_t iters,
 lbfs_status lbfs_step(lbfs_ctx* ctx, int32_t nsteps, lbfs_case_stats* out) {
     if (!ctx) return LBFS_EINVAL;
     if (nsteps < 0) return fail(ctx, LBFS_EINVAL, "nsteps must be >= 0");
+    CK(cudaSetDevice(ctx->cfg.device));
     if (ctx->dirty) {
         lbfs_status r = rebuild(ctx);
         if (r != LBFS_OK) return r;
     }
-    CK(cudaSetDevice(ctx->cfg.device));
     ctx->launches = 0;
     ctx->pot_fail = false;
     for (size_t c = 0; c < ctx->slots.size(); ++c)
@@ -1056,12 +1056,12 @@ int64_t lbfs_last_launch_count(const lbfs_ctx* ctx) { return ctx ? ctx->launches
 
 lbfs_status lbfs_autotune(lbfs_ctx* ctx, int32_t reps, int32_t* chosen, double* ms, int32_t n) {
     if (!ctx || reps < 1 || n < 0) return LBFS_EINVAL;
+    CK(cudaSetDevice(ctx->cfg.device));
     if (ctx->dirty) {
         lbfs_status r = rebuild(ctx);
         if (r != LBFS_OK) return r;
     }
     if (ctx->n_active == 0) return fail(ctx, LBFS_EINVAL, "no case defined");
-    CK(cudaSetDevice(ctx->cfg.device));
     cudaEvent_t a = take_event(ctx), b = take_event(ctx);
     int best = ctx->tile;
     double best_ms = 1e300;

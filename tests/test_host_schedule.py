@@ -215,3 +215,22 @@ def test_a_callers_allocator_need_not_align_to_a_quad(fake, monkeypatch, precisi
         s.close()
         stages = [w for w in fake.log() if w[0] == "stage"]
         assert len(stages) == 3 and not [w for w in stages if "misplaced" in w]
+
+
+@pytest.mark.parametrize("tune", [False, True])
+def test_lists_are_allocated_on_the_contexts_device(fake, tune):
+    """Whichever device the calling thread used last."""
+    fake.set("devices", 2)
+    second = lbfs.Solver(precision=lbfs.MIXED, max_cases=1, device=1)
+    second.set_case(0, _case())
+    first = lbfs.Solver(precision=lbfs.MIXED, max_cases=1, device=0)
+    fake.clear()
+    if tune:
+        second.autotune(1)
+    else:
+        second.step(1)
+    log = fake.log()
+    for s in (first, second):
+        s.close()
+    fake.set("devices", 1)
+    assert {w[3] for w in log if w[0] == "malloc"} == {"1"}
