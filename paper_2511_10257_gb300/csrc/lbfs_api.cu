@@ -256,14 +256,13 @@ lbfs_status resolve(lbfs_ctx* ctx, const lbfs_case_desc& d, CaseParams& P) {
 
 template <class R>
 void fill_phys(const CaseParams& P, PhysT<R>& q) {
-    q.rho_s = R(P.rho_s); q.rho_l = R(P.rho_l); q.rho_g = R(P.rho_g);
+    q.rho_s = R(P.rho_s); q.rho_g = R(P.rho_g);
     q.mu_s = R(P.mu_s); q.mu_l = R(P.mu_l); q.mu_g = R(P.mu_g);
     q.lam_s = R(P.lam_s); q.lam_l = R(P.lam_l); q.lam_g = R(P.lam_g);
-    q.cp_s = R(P.cp_s); q.cp_l = R(P.cp_l); q.cp_g = R(P.cp_g);
-    q.chi_s = R(P.chi_s); q.chi_l = R(P.chi_l); q.chi_g = R(P.chi_g);
-    q.beta = R(P.beta); q.kappa = R(P.kappa); q.Q_g = R(P.Q_g); q.cp_ref = R(P.cp_ref);
-    q.dts = R(P.dts); q.inv_dts = R(1.0 / P.dts); q.inv_cpref_dts = R(1.0 / (P.cp_ref * P.dts));
-    q.tau_g = R(0.5 + P.mobility / (P.Q_g * P.dts));
+    q.cp_s = R(P.cp_s); q.cp_g = R(P.cp_g);
+    q.chi_s = R(P.chi_s); q.chi_g = R(P.chi_g);
+    q.kappa = R(P.kappa); q.cp_ref = R(P.cp_ref);
+    q.inv_dts = R(1.0 / P.dts); q.inv_cpref_dts = R(1.0 / (P.cp_ref * P.dts));
     q.dt = R(P.dt); q.vol_ratio = R(P.vol_ratio); q.gravity = R(P.gravity); q.T_m = R(P.T_m); q.L = R(P.L);
     for (int w = 0; w < 4; ++w) q.wall_T[w] = R(P.wall_T[w]);
     q.wet = R(P.wet);
@@ -272,12 +271,12 @@ void fill_phys(const CaseParams& P, PhysT<R>& q) {
     q.Hes_lo = R(Hes - double(q.Hes_hi));
     q.L_hi = R(P.L);
     q.L_lo = R(P.L - double(q.L_hi));
-    q.rho_sg = q.rho_s - q.rho_g; q.rho_lg = q.rho_l - q.rho_g;
-    q.cp_sg = q.cp_s - q.cp_g; q.cp_lg = q.cp_l - q.cp_g;
+    q.rho_sg = q.rho_s - q.rho_g; q.rho_lg = R(P.rho_l) - q.rho_g;
+    q.cp_sg = q.cp_s - q.cp_g; q.cp_lg = R(P.cp_l) - q.cp_g;
     q.mu_sg = q.mu_s - q.mu_g; q.mu_lg = q.mu_l - q.mu_g;
-    q.lam_sg = q.lam_s - q.lam_g; q.lam_lg = q.lam_l - q.lam_g; q.chi_lg = q.chi_l - q.chi_g;
-    q.m_Qg = -q.Q_g; q.m_cp_ref3 = R(-P.cp_ref / 3.0);
-    q.cp_ref3 = R(P.cp_ref / 3.0); q.inv_cps = R(1.0 / P.cp_s);
+    q.lam_sg = q.lam_s - q.lam_g; q.lam_lg = q.lam_l - q.lam_g; q.chi_lg = R(P.chi_l) - q.chi_g;
+    q.m_Qg = -R(P.Q_g); q.m_cp_ref3 = R(-P.cp_ref / 3.0);
+    q.inv_cps = R(1.0 / P.cp_s);
     q.x_g = R(P.mobility / (P.Q_g * P.dts)); q.om_x_g = R(1) - q.x_g; q.beta2 = R(2.0 * P.beta); q.Qg3 = R(3.0 * P.Q_g);
     q.mhd = R(-0.5 * P.dts); q.off = R(0.5 * (0.5 - P.dts)); q.inv_dt = R(1.0 / P.dt);
 }

@@ -39,18 +39,18 @@ struct CaseParams {
 // so that no kernel converts FP64 parameters inside its inner loops.
 template <class R>
 struct PhysT {
-    R rho_s, rho_l, rho_g, mu_s, mu_l, mu_g, lam_s, lam_l, lam_g;
-    R cp_s, cp_l, cp_g, chi_s, chi_l, chi_g;
-    R beta, kappa, Q_g, cp_ref, dts, inv_dts, inv_cpref_dts, tau_g, dt, vol_ratio, gravity, T_m, L;
+    R rho_s, rho_g, mu_s, mu_l, mu_g, lam_s, lam_l, lam_g;
+    R cp_s, cp_g, chi_s, chi_g;
+    R kappa, cp_ref, inv_dts, inv_cpref_dts, dt, vol_ratio, gravity, T_m, L;
     R wall_T[4];
     R wet;
     // the thresholds H_es = C_p,s T_m and L of Eq. 8 as (hi, lo) pairs of R: the exact
     // FP64 value is hi + lo to FP32-pair accuracy (lo = 0 in FP64)
     R Hes_hi, Hes_lo, L_hi, L_lo;
-    // what the stage kernel uses of the above, formed once: property differences g_s - g_g
-    // and g_l - g_g, C_p,ref/3, 1/C_p,s, tau_g - 1/2, 2 beta, 3 Q_g, -dts/2, (1/2 - dts)/2, 1/dt
+    // formed once: property differences g_s - g_g and g_l - g_g, -Q_g, -C_p,ref/3, 1/C_p,s,
+    // tau_g - 1/2 and one minus it, 2 beta, 3 Q_g, -dts/2, (1/2 - dts)/2, 1/dt
     R rho_sg, rho_lg, cp_sg, cp_lg, mu_sg, mu_lg, lam_sg, lam_lg, chi_lg;
-    R m_Qg, m_cp_ref3, om_x_g, cp_ref3, inv_cps, x_g, beta2, Qg3, mhd, off, inv_dt;
+    R m_Qg, m_cp_ref3, om_x_g, inv_cps, x_g, beta2, Qg3, mhd, off, inv_dt;
 };
 
 // p, rho c_s^2 u, rho c_s^2 v and C of one cell: one vector load or store
@@ -90,7 +90,7 @@ struct DevCase {
     void* W[3];       // Quad<R>: p, rho c_s^2 u, rho c_s^2 v, C
     void* phi;        // potential read by the stage kernel (R); FP64 mode: the master
     double* phi64;    // FP64 mode: the master potential (== phi); mixed: unused
-    double* phi_prev64;  // FP64 mode: the previous step's potential; mixed: unused
+    double* phi_prev64;  // FP64 mode: the potentials of the last step and of the one before it; mixed: unused
     float* phi_lo;    // mixed: low word of the master potential phi + phi_lo (FP32 pair)
     void* Fs_prev;    // R: F_s of the previous step, replaced by F_s^n in stage 1
     void* Sdot;       // R: lagged dF_s/dt of the current step, written by stage 1
@@ -139,19 +139,6 @@ struct StageCase {
 struct TileRef {
     int case_id, x0, y0, slot;
 };
-
-// ---------------------------------------------------------------------------
-// D2Q9 (Eq. 14, Fig. 1) with the textbook weights 4/9, 1/9, 1/36.
-// ---------------------------------------------------------------------------
-__host__ __device__ constexpr int d2q9_ex(int a) {
-    return a == 1 || a == 5 || a == 8 ? 1 : (a == 3 || a == 6 || a == 7 ? -1 : 0);
-}
-__host__ __device__ constexpr int d2q9_ey(int a) {
-    return a == 2 || a == 5 || a == 6 ? 1 : (a == 4 || a == 7 || a == 8 ? -1 : 0);
-}
-__host__ __device__ constexpr double d2q9_w(int a) {
-    return a == 0 ? 4.0 / 9.0 : (a <= 4 ? 1.0 / 9.0 : 1.0 / 36.0);
-}
 
 // Eq. 11 mixture: F_s g_s + (1 - F_s) C g_l + (1 - F_s)(1 - C) g_g
 template <class R>
@@ -347,12 +334,6 @@ template <>
 struct HeStore<float> {
     using T = float2;
 };
-template <class S>
-__device__ __forceinline__ S he_zero();
-template <>
-__device__ __forceinline__ double he_zero<double>() { return 0.0; }
-template <>
-__device__ __forceinline__ float2 he_zero<float2>() { return make_float2(0.0f, 0.0f); }
 __device__ __forceinline__ double he_value(double h) { return h; }
 __device__ __forceinline__ double he_value(float2 h) { return (double)h.x + (double)h.y; }
 template <class R>
@@ -386,11 +367,6 @@ __device__ __forceinline__ void phi_set(const DevCase* dc, size_t k, double v) {
         static_cast<float*>(dc->phi)[k] = h;
         dc->phi_lo[k] = l;
     }
-}
-
-template <class R>
-__device__ __forceinline__ R load(const void* base, size_t idx) {
-    return static_cast<const R*>(base)[idx];
 }
 
 }  // namespace lbfs
