@@ -544,8 +544,8 @@ int phased_cycles(int prec, int cases) {
 // them in one launch needs all its blocks to run at once and cannot have that on this stream
 bool launched_cycles(const lbfs_ctx* ctx) { return ctx->cfg.mg_plain_cycles || ctx->coop == 0; }
 
-// The potential of the current state: in FP64 a warm step starts from the linearly
-// extrapolated potential; then the step's first residual and check, then refinement cycles
+// The potential of the current state: in FP64 a warm step starts from the potential
+// extrapolated in time; then the step's first residual and check, then refinement cycles
 // (V-cycle, correction, residual of the corrected potential, check), which the checks end on the
 // device, so a step whose start already meets mg_tol runs none and no host round trip is
 // made.  At most mg_warm_cycles cycles, or mg_max_cycles after a state was set (pot_fresh); a

@@ -128,7 +128,8 @@ __global__ void k_derive(const DevCase* __restrict__ dc, uint32_t mask, double* 
 // The bound's margin of 1e-3 is far above its rounding; cells outside the range in which that
 // is so (cancelling densities, C > 2, NaN) are always evaluated.
 // One thread a column, serial over the rows in FP64, had 8 blocks on 1024 x 512 and took about
-// half of a monitoring pass (diagnostics and six derived fields): 1157 us, now 590.
+// half of a monitoring pass (diagnostics and six derived fields): 1157 us, now 580 to 680 with
+// the host link's spread.
 constexpr int kDiagWarps = 32, kDiagAhead = 4;
 
 template <class R>

@@ -55,7 +55,7 @@ cudaError_t launch_mg_tail(int prec, const DevCase* cases, const int* case_ids, 
                            cudaStream_t st);
 // the coarsest level of the other cases
 cudaError_t launch_mg_coarsest(const DevCase* cases, const int* case_ids, int ncases, int max_cells, cudaStream_t st);
-// FP64 only: the linearly extrapolated warm start of the potential
+// FP64 only: the warm start of the potential, extrapolated in time (linearly, later through three points)
 cudaError_t launch_mg_extrapolate(const DevCase* cases, const TileRef* tiles, int n, cudaStream_t st);
 // fused V-cycle legs over 32 x 16 tiles of one level (kFusedTX x kFusedTY), or over
 // 16 x 8 tiles (small != 0) on a level whose 32 x 16 tiles would not fill the GPU

@@ -433,14 +433,14 @@ struct RowQ {
 //
 // Bound by instruction issue and the latency of one row's chain (FP32: 59 % of the issue slots
 // busy, 44 % of the FMA pipe; HBM at a third), in FP64 by the FP64 pipe.  A marching strip derives
-// each cell 1.23 times instead of a 32 x 8 tile's 2.08, forms a cell's side sums once for both
-// its faces instead of once per face, and reads a face's operands from registers and shuffles
-// instead of 54 shared-memory loads: 4096x2048, mixed, 1637 -> 853 thread instructions per cell
-// and 0.52 -> 0.28 ms a launch; FP64 18.6 -> 11.3 ms; 1024x512, mixed, 64 -> 33 us.  At 168
-// registers 12 warps an SM; 16 warps (128 registers) spill and take 0.50 ms, two columns per
-// lane (255 registers, 8 warps) 0.37-0.43 ms.  Strips away from walls and wraps run without any of
-// their logic (0.35 -> 0.30 ms), coefficients from the constant bank save 4 %, copies four
-// rows ahead 7 %.
+// each cell (rows + 4)/rows x 32/26 times, 1.44 with 24 rows (6.2 with one), instead of a 32 x 8
+// tile's 2.08, forms a cell's side sums once for both its faces instead of once per face, and
+// reads a face's operands from registers and shuffles instead of 54 shared-memory loads:
+// 4096x2048, mixed, 1637 -> 851 thread instructions per cell and 0.52 -> 0.28 ms a launch; FP64
+// 18.6 -> 11.3 ms; 1024x512, mixed, 64 -> 33 us.  At 168 registers 12 warps an SM; 16 warps (128
+// registers) spill and take 0.50 ms, two columns per lane (255 registers, 8 warps) 0.37-0.43 ms.
+// Strips away from walls and wraps run without any of their logic (0.35 -> 0.30 ms),
+// coefficients from the constant bank save 4 %, copies four rows ahead 7 %.
 template <class R, int STAGE, bool HALF, bool UNI>
 __global__ void __launch_bounds__(32, sizeof(R) == 4 ? 12 : 4)
 stage_kernel(const StageCase<R>* __restrict__ cases, const TileRef* __restrict__ tiles, int rows,
