@@ -3,6 +3,7 @@ allocates, copies, waits for and launches can be followed on a machine without a
 failing call can be faked.  Kernels do nothing there."""
 import ctypes as ct
 import os
+import shutil
 import subprocess
 
 from paper_2511_10257_gb300 import build as B
@@ -13,7 +14,8 @@ SOURCES = [os.path.join(B.CSRC, f) for f in ("lbfs_api.cu", "lbfs_potential.cu",
 
 def build(folder) -> str:
     """compile (device code only as far as PTX, unoptimised) and link; the path of the library"""
-    inc = ["-I", os.path.join(B.ROOT, "include"), "-I", B.CSRC, "-I", os.path.join(os.path.dirname(B.nvcc()), "..", "include")]
+    toolkit = os.path.dirname(os.path.dirname(shutil.which(B.nvcc()) or B.nvcc()))
+    inc = ["-I", os.path.join(B.ROOT, "include"), "-I", B.CSRC, "-I", os.path.join(toolkit, "include")]
     nvcc = [B.nvcc(), "-gencode", "arch=compute_103a,code=compute_103a", "-O1", "-Xcicc", "-O0", "-Xcompiler", "-fPIC"]
     procs, objs = [], []
     for src in SOURCES + [os.path.join(HERE, "host", f) for f in ("fake_stage.cu", "fake_cuda.cpp")]:

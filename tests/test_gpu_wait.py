@@ -17,6 +17,9 @@ def test_a_wait_that_runs_out_is_an_error_status(precision):
     s.set_case(0, c)
     status, _ = s.step(1, raise_on_error=False)
     assert status == lbfs.ETIMEOUT
+    for n in (1, 3):   # the context launches its cycles from now on, and its checks sum whole residuals
+        st = s.step(n)[0]
+        assert 0.0 < st["pot_resid_max"] <= s.mg_tol_used()
     s.close()
     out = []
     for plain in (False, True):
